@@ -33,6 +33,7 @@
 #include <atomic>
 
 #include "gk_internal.cuh"
+#include "stripe.cuh"
 
 namespace gk {
 
@@ -651,24 +652,56 @@ __device__ __forceinline__ void deferred_finish(const FilterArgs &a, uint32_t K,
   }
 }
 
-// Read and window planes of a loaded pair, zero past m.
+// Window planes of a loaded pair, zero past m.
 template <int W>
-__device__ __forceinline__ void pair_planes(const PairData<W> &x, uint32_t (&rh)[W], uint32_t (&rl)[W],
-                                            uint32_t (&gh)[W], uint32_t (&gl)[W]) {
+__device__ __forceinline__ void window_planes(const PairData<W> &x, uint32_t (&gh)[W], uint32_t (&gl)[W]) {
   const uint32_t tail = x.m - 32u * (W - 1);
   const uint32_t lastmask = tail >= 32 ? 0xffffffffu : ((1u << tail) - 1u);
   const uint32_t sh = x.off & 31;
 #pragma unroll
   for (int w = 0; w < W; ++w) {
-    rh[w] = x.r[w].x;
-    rl[w] = x.r[w].y;
     gh[w] = __funnelshift_r(x.g[w].x, x.g[w + 1].x, sh);
     gl[w] = __funnelshift_r(x.g[w].y, x.g[w + 1].y, sh);
   }
-  rh[W - 1] &= lastmask;
-  rl[W - 1] &= lastmask;
   gh[W - 1] &= lastmask;
   gl[W - 1] &= lastmask;
+}
+
+// Read planes of a loaded pair, zero past m.
+template <int W>
+__device__ __forceinline__ void read_planes(const PairData<W> &x, uint32_t (&rh)[W], uint32_t (&rl)[W]) {
+  const uint32_t tail = x.m - 32u * (W - 1);
+  const uint32_t lastmask = tail >= 32 ? 0xffffffffu : ((1u << tail) - 1u);
+#pragma unroll
+  for (int w = 0; w < W; ++w) {
+    rh[w] = x.r[w].x;
+    rl[w] = x.r[w].y;
+  }
+  rh[W - 1] &= lastmask;
+  rl[W - 1] &= lastmask;
+}
+
+template <int W>
+__device__ __forceinline__ void pair_planes(const PairData<W> &x, uint32_t (&rh)[W], uint32_t (&rl)[W],
+                                            uint32_t (&gh)[W], uint32_t (&gl)[W]) {
+  read_planes<W>(x, rh, rl);
+  window_planes<W>(x, gh, gl);
+}
+
+// The same as S stripes.
+template <int W, int S>
+__device__ __forceinline__ void striped_window(const PairData<W> &x, uint32_t (&gh)[S], uint32_t (&gl)[S]) {
+  uint32_t h[W], l[W];
+  window_planes<W>(x, h, l);
+  stripe_linear<W, S>(h, gh);
+  stripe_linear<W, S>(l, gl);
+}
+template <int W, int S>
+__device__ __forceinline__ void striped_read(const PairData<W> &x, uint32_t (&rh)[S], uint32_t (&rl)[S]) {
+  uint32_t h[W], l[W];
+  read_planes<W>(x, h, l);
+  stripe_linear<W, S>(h, rh);
+  stripe_linear<W, S>(l, rl);
 }
 
 template <int W, bool DIRECT = false>
@@ -685,10 +718,13 @@ __device__ __forceinline__ uint32_t filter_loaded_deferred(const FilterArgs &a, 
 // 6 fit 4 and 3 blocks without spilling (at 150 bp, e = 0..2, 4 blocks run
 // 9-18% faster than 2).  The compacting loop stages its words with cp.async
 // and carries a chunk pipeline, so it keeps fewer resident warps.
-template <int W, bool COMPACT>
+// The striped sweep needs 56 (S <= 4), 72 (S = 5), 93 (S = 8) and 128 (S =
+// 11) registers.
+template <int W, bool COMPACT, int S = 0>
 struct MinBlocks {
   static constexpr int value =
-      COMPACT ? (W <= 2 ? 5 : (W <= 4 ? 4 : (W <= 6 ? 3 : (W <= 8 ? 2 : 1))))
+      S > 0 ? (S <= 4 ? 4 : (S == 5 ? 3 : 2))
+      : COMPACT ? (W <= 2 ? 5 : (W <= 4 ? 4 : (W <= 6 ? 3 : (W <= 8 ? 2 : 1))))
               : (W <= 2 ? 6 : (W <= 4 ? 5 : (W == 5 ? 4 : (W == 6 ? 3 : (W <= 8 ? 2 : 1)))));
 };
 
@@ -741,18 +777,17 @@ __device__ __forceinline__ void write_count(const FilterArgs &a, uint64_t p, uin
 // Threshold sweep of one loaded pair (VARIANT 3): thresholds e = a.fixed_e ..
 // a.sweep_hi have shift counts K = min(e, m-1); the shift loop runs once to
 // the largest and the results of each K go to its rows (every e >= m-1
-// shares K = m-1).
-template <int W>
+// shares K = m-1).  S > 0: striped in S words, else linear with deferred
+// erosion.
+template <int W, int S>
 __device__ __forceinline__ void sweep_and_write(const FilterArgs &a, uint64_t p, const PairData<W> &x) {
-  uint32_t rh[W], rl[W], gh[1][W], gl[1][W], count[1];
-  pair_planes<W>(x, rh, rl, gh[0], gl[0]);
   const uint32_t e_lo = a.fixed_e, e_hi = a.sweep_hi, kmax = x.m - 1;
   const uint32_t Klo = min(e_lo, kmax), Khi = min(e_hi, kmax);
   // The common case (K in e_lo..e_hi, below m-1) writes one row: its
   // pointers advance by a row per shift count.
   uint8_t *acc_row = a.accept + p;
   uint16_t *ed_row = a.edits + p;
-  deferred_sweep_counts<W, 1>(a, x.m, Khi, rh, rl, gh, gl, count, Klo, [&](uint32_t K, const uint32_t (&c)[1]) {
+  auto emit = [&](uint32_t K, const uint32_t (&c)[1]) {
     if (!a.result_byte && K >= e_lo && K < kmax) {
       *acc_row = c[0] <= K;
       *ed_row = (uint16_t)c[0];
@@ -762,13 +797,26 @@ __device__ __forceinline__ void sweep_and_write(const FilterArgs &a, uint64_t p,
     }
     const uint32_t first = K > e_lo ? K : e_lo, last = K == kmax ? e_hi : K;
     for (uint32_t e = first; e <= last; ++e) write_count(a, p + (uint64_t)(e - e_lo) * a.out_stride, c[0], e);
-  });
+  };
+  if constexpr (S > 0) {
+    uint32_t rh[S], rl[S], gh[1][S], gl[1][S];
+    striped_read<W, S>(x, rh, rl);
+    striped_window<W, S>(x, gh[0], gl[0]);
+    if (x.m % S == 0)
+      striped_exact<W, S, 1, true>(x.m, Klo, Khi, a.count_mode, rh, rl, gh, gl, emit);
+    else
+      striped_exact<W, S, 1, false>(x.m, Klo, Khi, a.count_mode, rh, rl, gh, gl, emit);
+  } else {
+    uint32_t rh[W], rl[W], gh[1][W], gl[1][W], count[1];
+    pair_planes<W>(x, rh, rl, gh[0], gl[0]);
+    deferred_sweep_counts<W, 1>(a, x.m, Khi, rh, rl, gh, gl, count, Klo, emit);
+  }
 }
 
-template <int W, int VARIANT>
+template <int W, int VARIANT, int S = 0>
 __device__ __forceinline__ void filter_and_write(const FilterArgs &a, uint64_t p, const PairData<W> &x) {
   if constexpr (VARIANT == 3) {
-    sweep_and_write<W>(a, p, x);
+    sweep_and_write<W, S>(a, p, x);
   } else {
     const uint32_t count = VARIANT == 4   ? filter_loaded_deferred<W, true>(a, x)
                            : VARIANT == 2 ? filter_loaded_deferred<W>(a, x)
@@ -849,7 +897,8 @@ constexpr size_t compact_smem_bytes() {
 
 // VARIANT 0: any thresholds; 1: every shift count of the launch is < 32;
 // 2: edge OR on and one threshold in 2..30, deferred erosion; 3: edge OR on,
-// a sweep of thresholds up to 30, deferred erosion (sweep_and_write).
+// a sweep of thresholds up to 30 (sweep_and_write; striped in S words or, S =
+// 0, linear).
 //
 // COMPACT false: one thread per pair.  COMPACT true (inputs with many
 // undefined pairs): persistent warps take 32 pairs at a time (their ids
@@ -860,8 +909,8 @@ constexpr size_t compact_smem_bytes() {
 // lane idles next to an undefined pair and the word loads of one batch hide
 // behind the arithmetic of the other.  Dynamic shared memory:
 // compact_smem_bytes<W>().
-template <int W, int VARIANT, bool COMPACT>
-__global__ void __launch_bounds__(kFilterThreads, MinBlocks<W, COMPACT>::value) filter_kernel(const FilterArgs a) {
+template <int W, int VARIANT, bool COMPACT, int S = 0>
+__global__ void __launch_bounds__(kFilterThreads, MinBlocks<W, COMPACT, S>::value) filter_kernel(const FilterArgs a) {
   if (!COMPACT) {
     const uint64_t p = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x;
     const bool active = p < a.n_pairs;
@@ -878,7 +927,7 @@ __global__ void __launch_bounds__(kFilterThreads, MinBlocks<W, COMPACT>::value) 
       write_trivial<VARIANT == 3>(a, p, status);
       return;
     }
-    filter_and_write<W, VARIANT>(a, p, cur);
+    filter_and_write<W, VARIANT, S>(a, p, cur);
     return;
   }
   extern __shared__ uint2 stage_all[];
@@ -919,7 +968,7 @@ __global__ void __launch_bounds__(kFilterThreads, MinBlocks<W, COMPACT>::value) 
     for (int w = 0; w < W; ++w) x.r[w] = sb[w * 32 + lane];
 #pragma unroll
     for (int w = 0; w <= W; ++w) x.g[w] = sb[(W + w) * 32 + lane];
-    filter_and_write<W, VARIANT>(a, pend_p, x);
+    filter_and_write<W, VARIANT, S>(a, pend_p, x);
   };
   for (;; c += n_warps) {
     const bool more = c < n_chunks;
@@ -1012,8 +1061,7 @@ struct MinBlocks2 {
   static constexpr int value = 4;
 };
 
-// Deferred erosion (VARIANT 2, or the sweep, VARIANT 3), two pairs per
-// thread: pairs 2t and 2t+1.  When both are filtered and share their read
+// Deferred erosion (VARIANT 2), two pairs per thread: pairs 2t and 2t+1.  When both are filtered and share their read
 // (the candidates of one read usually sit next to each other), the read is
 // loaded once and its shifted copies serve both windows: a shift step costs
 // about 13W integer operations per pair instead of 15W.  Otherwise each pair
@@ -1041,77 +1089,24 @@ __global__ void __launch_bounds__(kFilterThreads, MinBlocks2<W>::value) filter_p
   }
   const int s0 = act0 ? pair_status<W>(a, x0) : -1;
   const int s1 = act1 ? pair_status<W>(a, x1) : -1;
-  if (s0 > 0) write_trivial<VARIANT == 3>(a, p0, s0);
-  if (s1 > 0) write_trivial<VARIANT == 3>(a, p1, s1);
+  if (s0 > 0) write_trivial(a, p0, s0);
+  if (s1 > 0) write_trivial(a, p1, s1);
   if (s0 == 0 && s1 == 0 && x0.rid == x1.rid) {
     uint32_t rh[W], rl[W], gh[2][W], gl[2][W], count[2];
     pair_planes<W>(x0, rh, rl, gh[0], gl[0]);
-    {
-      const uint32_t tail = a.m - 32u * (W - 1);
-      const uint32_t lastmask = tail >= 32 ? 0xffffffffu : ((1u << tail) - 1u);
-      const uint32_t sh = x1.off & 31;
-#pragma unroll
-      for (int w = 0; w < W; ++w) {
-        gh[1][w] = __funnelshift_r(x1.g[w].x, x1.g[w + 1].x, sh);
-        gl[1][w] = __funnelshift_r(x1.g[w].y, x1.g[w + 1].y, sh);
-      }
-      gh[1][W - 1] &= lastmask;
-      gl[1][W - 1] &= lastmask;
-    }
-    if constexpr (VARIANT == 3) {
-      const uint32_t e_lo = a.fixed_e, e_hi = a.sweep_hi, kmax = a.m - 1;
-      // Pairs 2t and 2t+1 are adjacent in every row: one 2-byte and one
-      // 4-byte store per threshold when the rows keep that alignment.
-      const bool pack = (((uintptr_t)a.accept | (a.result_byte ? 0u : (uintptr_t)a.edits)) & 3u) == 0 &&
-                        (a.out_stride & 1u) == 0;
-      // The common case (K in e_lo..e_hi, below m-1) writes one row: its
-      // accept and count pointers advance by a row per shift count.
-      uint8_t *acc_row = a.accept + p0;
-      uint16_t *ed_row = a.edits + p0;
-      deferred_sweep_counts<W, 2>(a, a.m, min(e_hi, kmax), rh, rl, gh, gl, count, min(e_lo, kmax),
-                                  [&](uint32_t K, const uint32_t (&c)[2]) {
-                                    if (pack && !a.result_byte && K >= e_lo && K < kmax) {
-                                      *reinterpret_cast<uint32_t *>(ed_row) = c[0] | (c[1] << 16);
-                                      *reinterpret_cast<uint16_t *>(acc_row) =
-                                          (uint16_t)((c[0] <= K ? 1u : 0u) | (c[1] <= K ? 0x100u : 0u));
-                                      acc_row += a.out_stride;
-                                      ed_row += a.out_stride;
-                                      return;
-                                    }
-                                    const uint32_t first = K > e_lo ? K : e_lo, last = K == kmax ? e_hi : K;
-                                    for (uint32_t e = first; e <= last; ++e) {
-                                      const uint64_t o = (uint64_t)(e - e_lo) * a.out_stride;
-                                      if (pack) {
-                                        uint32_t b0, b1;
-                                        if (a.result_byte) {
-                                          b0 = min(c[0], GK_RESULT_MAX_COUNT);
-                                          b1 = min(c[1], GK_RESULT_MAX_COUNT);
-                                        } else {
-                                          b0 = c[0] <= e;
-                                          b1 = c[1] <= e;
-                                          *reinterpret_cast<uint32_t *>(a.edits + o + p0) = c[0] | (c[1] << 16);
-                                        }
-                                        *reinterpret_cast<uint16_t *>(a.accept + o + p0) = (uint16_t)(b0 | (b1 << 8));
-                                      } else {
-                                        write_count(a, p0 + o, c[0], e);
-                                        write_count(a, p1 + o, c[1], e);
-                                      }
-                                    }
-                                  });
+    window_planes<W>(x1, gh[1], gl[1]);
+    const uint32_t K = KC >= 0 ? (uint32_t)KC : min(a.fixed_e, a.m - 1);
+    deferred_counts<W, 2, (KC >= 0)>(a, a.m, K, rh, rl, gh, gl, count);
+    // The two pairs are adjacent: one 2-byte accept store and one 4-byte
+    // count store when the buffers allow it.
+    if (!a.result_byte && ((uintptr_t)a.accept & 1u) == 0 && ((uintptr_t)a.edits & 3u) == 0) {
+      const uint32_t e = a.fixed_e;
+      *reinterpret_cast<uint32_t *>(a.edits + p0) = count[0] | (count[1] << 16);
+      *reinterpret_cast<uint16_t *>(a.accept + p0) =
+          (uint16_t)((count[0] <= e ? 1u : 0u) | (count[1] <= e ? 0x100u : 0u));
     } else {
-      const uint32_t K = KC >= 0 ? (uint32_t)KC : min(a.fixed_e, a.m - 1);
-      deferred_counts<W, 2, (KC >= 0)>(a, a.m, K, rh, rl, gh, gl, count);
-      // The two pairs are adjacent: one 2-byte accept store and one 4-byte
-      // count store when the buffers allow it.
-      if (!a.result_byte && ((uintptr_t)a.accept & 1u) == 0 && ((uintptr_t)a.edits & 3u) == 0) {
-        const uint32_t e = a.fixed_e;
-        *reinterpret_cast<uint32_t *>(a.edits + p0) = count[0] | (count[1] << 16);
-        *reinterpret_cast<uint16_t *>(a.accept + p0) =
-            (uint16_t)((count[0] <= e ? 1u : 0u) | (count[1] <= e ? 0x100u : 0u));
-      } else {
-        write_count(a, p0, count[0], a.fixed_e);
-        write_count(a, p1, count[1], a.fixed_e);
-      }
+      write_count(a, p0, count[0], a.fixed_e);
+      write_count(a, p1, count[1], a.fixed_e);
     }
   } else {
     if (s0 == 0) filter_and_write<W, VARIANT>(a, p0, x0);
@@ -1119,17 +1114,117 @@ __global__ void __launch_bounds__(kFilterThreads, MinBlocks2<W>::value) filter_p
   }
 }
 
+// The threshold sweep, two pairs per thread (2t and 2t+1): when both are
+// filtered and share their read, its shifted copies and their masks serve both
+// windows, and each threshold's two results go out as one 2-byte and one
+// 4-byte store.  Rows are addressed as a block's base plus a 32-bit offset, so
+// that their advance is scalar work.  Pairs that do not share are loaded anew,
+// one after the other (keeping both over the shared form's registers spills).
+// S: stripes, or 0 for the linear form.  Blocks per SM: 64 registers hold S <=
+// 4 (3 blocks measured 1% slower at 100 bp), 80 S = 5 (2 blocks 7% slower at
+// 150 bp; one pair per thread 12% slower).
+template <int W, int S>
+__global__ void __launch_bounds__(kFilterThreads, S == 5 ? 3 : 4) sweep_pair2_kernel(const FilterArgs a) {
+  const uint64_t base = blockIdx.x * (uint64_t)(2 * kFilterThreads);
+  const uint32_t lo = 2 * threadIdx.x;
+  const uint64_t p0 = base + lo, p1 = p0 + 1;
+  const bool act0 = p0 < a.n_pairs, act1 = p1 < a.n_pairs;
+  PairData<W> x0, x1;
+  x0.status = x1.status = 0;
+  if (act0) load_pair<W>(a, p0, x0);
+  if (act1) load_pair<W>(a, p1, x1, act0 ? &x0 : nullptr);
+  if (a.err_count) {
+    const unsigned b0 = __ballot_sync(0xffffffffu, act0 && x0.status == 2);
+    const unsigned b1 = __ballot_sync(0xffffffffu, act1 && x1.status == 2);
+    if ((b0 | b1) && (threadIdx.x & 31) == 0) atomicAdd(a.err_count, (unsigned)(__popc(b0) + __popc(b1)));
+  }
+  const int s0 = act0 ? pair_status<W>(a, x0) : -1;
+  const int s1 = act1 ? pair_status<W>(a, x1) : -1;
+  if (s0 > 0) write_trivial<true>(a, p0, s0);
+  if (s1 > 0) write_trivial<true>(a, p1, s1);
+  if (s0 == 0 && s1 == 0 && x0.rid == x1.rid) {
+    const uint32_t e_lo = a.fixed_e, e_hi = a.sweep_hi, kmax = a.m - 1;
+    const uint32_t Klo = min(e_lo, kmax), Khi = min(e_hi, kmax);
+    // Pairs 2t and 2t+1 are adjacent in every row: packed stores when the
+    // rows keep that alignment.
+    const bool pack = (((uintptr_t)a.accept | (a.result_byte ? 0u : (uintptr_t)a.edits)) & 3u) == 0 &&
+                      (a.out_stride & 1u) == 0;
+    const bool one_row = pack && !a.result_byte;
+    // The common case (K in e_lo..e_hi, below m-1) writes one row.
+    uint8_t *acc_row = a.accept + base;
+    uint16_t *ed_row = a.edits + base;
+    auto emit = [&](uint32_t K, const uint32_t (&c)[2]) {
+      if (one_row && K < kmax) {
+        *reinterpret_cast<uint32_t *>(ed_row + lo) = c[0] | (c[1] << 16);
+        *reinterpret_cast<uint16_t *>(acc_row + lo) =
+            (uint16_t)((c[0] <= K ? 1u : 0u) | (c[1] <= K ? 0x100u : 0u));
+        acc_row += a.out_stride;
+        ed_row += a.out_stride;
+        return;
+      }
+      const uint32_t first = K > e_lo ? K : e_lo, last = K == kmax ? e_hi : K;
+      for (uint32_t e = first; e <= last; ++e) {
+        const uint64_t o = (uint64_t)(e - e_lo) * a.out_stride;
+        if (pack) {
+          uint32_t b0, b1;
+          if (a.result_byte) {
+            b0 = min(c[0], GK_RESULT_MAX_COUNT);
+            b1 = min(c[1], GK_RESULT_MAX_COUNT);
+          } else {
+            b0 = c[0] <= e;
+            b1 = c[1] <= e;
+            *reinterpret_cast<uint32_t *>(a.edits + o + p0) = c[0] | (c[1] << 16);
+          }
+          *reinterpret_cast<uint16_t *>(a.accept + o + p0) = (uint16_t)(b0 | (b1 << 8));
+        } else {
+          write_count(a, p0 + o, c[0], e);
+          write_count(a, p1 + o, c[1], e);
+        }
+      }
+    };
+    if constexpr (S > 0) {
+      uint32_t rh[S], rl[S], gh[2][S], gl[2][S];
+      striped_read<W, S>(x0, rh, rl);
+      striped_window<W, S>(x0, gh[0], gl[0]);
+      striped_window<W, S>(x1, gh[1], gl[1]);
+      if (a.m % S == 0)
+        striped_exact<W, S, 2, true>(a.m, Klo, Khi, a.count_mode, rh, rl, gh, gl, emit);
+      else
+        striped_exact<W, S, 2, false>(a.m, Klo, Khi, a.count_mode, rh, rl, gh, gl, emit);
+    } else {
+      uint32_t rh[W], rl[W], gh[2][W], gl[2][W], count[2];
+      pair_planes<W>(x0, rh, rl, gh[0], gl[0]);
+      window_planes<W>(x1, gh[1], gl[1]);
+      deferred_sweep_counts<W, 2>(a, a.m, Khi, rh, rl, gh, gl, count, Klo, emit);
+    }
+  } else {
+#pragma unroll 1
+    for (int j = 0; j < 2; ++j) {
+      if ((j ? s1 : s0) != 0) continue;
+      load_pair<W>(a, p0 + j, x0);
+      sweep_and_write<W, S>(a, p0 + j, x0);
+    }
+  }
+}
+
 // Launches one instantiation of the plain filter over a.n_pairs pairs.
-template <int W, int VARIANT>
+template <int W, int VARIANT, int S = 0>
 cudaError_t launch_filter_variant(const FilterArgs &a, cudaStream_t stream) {
   unsigned blocks = (unsigned)((a.n_pairs + kFilterThreads - 1) / kFilterThreads);
   if (a.compact == 0) {
-    // Two pairs per thread for W <= 4 only: at W = 5 (2 blocks per SM with
-    // its registers unspilled) it measured 40% slower at e = 2, 150 bp.
-    if constexpr ((VARIANT == 2 || VARIANT == 3 || VARIANT == 4) && W <= 4) {
+    const uint64_t threads = (a.n_pairs + 1) / 2;
+    const unsigned grid = (unsigned)((threads + kFilterThreads - 1) / kFilterThreads);
+    // Two pairs per thread for W <= 4 and the striped sweep of W = 5: the
+    // linear form at W = 5 (2 blocks per SM with its registers unspilled)
+    // measured 40% slower at e = 2, 150 bp.
+    if constexpr (VARIANT == 3 && (W <= 4 || S == 5)) {
       if (a.m > 0) {
-        const uint64_t threads = (a.n_pairs + 1) / 2;
-        const unsigned grid = (unsigned)((threads + kFilterThreads - 1) / kFilterThreads);
+        sweep_pair2_kernel<W, S><<<grid, kFilterThreads, 0, stream>>>(a);
+        return cudaGetLastError();
+      }
+    }
+    if constexpr ((VARIANT == 2 || VARIANT == 4) && W <= 4) {
+      if (a.m > 0) {
         if constexpr (VARIANT == 4) {
           // shift count = the threshold, 0..2, below m (checked by the caller)
           switch (a.fixed_e) {
@@ -1147,7 +1242,7 @@ cudaError_t launch_filter_variant(const FilterArgs &a, cudaStream_t stream) {
     if constexpr (VARIANT == 4) {
       return cudaErrorInvalidValue;  // VARIANT 4 is the two-pair kernel only
     } else {
-      filter_kernel<W, VARIANT, false><<<blocks, kFilterThreads, 0, stream>>>(a);
+      filter_kernel<W, VARIANT, false, S><<<blocks, kFilterThreads, 0, stream>>>(a);
       return cudaGetLastError();
     }
   }
@@ -1167,14 +1262,14 @@ cudaError_t launch_filter_variant(const FilterArgs &a, cudaStream_t stream) {
   const size_t smem = compact_smem_bytes<W>();
   int blocks_per_sm = per_sm[dev].load(std::memory_order_acquire);
   if (blocks_per_sm == 0) {
-    err = cudaFuncSetAttribute(filter_kernel<W, VARIANT, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    err = cudaFuncSetAttribute(filter_kernel<W, VARIANT, true, S>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                (int)smem);
     if (err != cudaSuccess) return err;
     int count = 0;
     err = cudaDeviceGetAttribute(&count, cudaDevAttrMultiProcessorCount, dev);
     if (err != cudaSuccess) return err;
     int n = 0;
-    err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, filter_kernel<W, VARIANT, true>, kFilterThreads, smem);
+    err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, filter_kernel<W, VARIANT, true, S>, kFilterThreads, smem);
     if (err != cudaSuccess) return err;
     blocks_per_sm = n < 1 ? 1 : n;
     sms[dev].store(count, std::memory_order_relaxed);
@@ -1182,8 +1277,29 @@ cudaError_t launch_filter_variant(const FilterArgs &a, cudaStream_t stream) {
   }
   const uint64_t wave = 4ull * (uint64_t)sms[dev].load(std::memory_order_relaxed) * (uint64_t)blocks_per_sm;
   if (blocks > wave) blocks = (unsigned)wave;
-  filter_kernel<W, VARIANT, true><<<blocks, kFilterThreads, smem, stream>>>(a);
+  filter_kernel<W, VARIANT, true, S><<<blocks, kFilterThreads, smem, stream>>>(a);
   return cudaGetLastError();
+  }
+}
+
+// Launches the threshold sweep over reads of W = ceil(m/32) words: striped
+// where the stripes hold the read (stripe_limit) and beat the linear form.
+// Measured on GB300, launches alone, linear -> striped: 76 bp (S = 3) at e =
+// 0..8 0.230 -> 0.166 ms; 200 bp (S = 8) at 0..20 0.599 -> 0.443; 300 bp (S =
+// 11) at 0..30 1.146 -> 0.958; 100, 150 and 250 bp beside striped_exact.  W =
+// 1 needs one linear word and three stripes; from W = 11 on the stripes spill.
+template <int W>
+cudaError_t launch_sweep(const FilterArgs &a, cudaStream_t stream) {
+  if constexpr (W == 1 || W > 10) {
+    return launch_filter_variant<W, 3>(a, stream);
+  } else {
+    constexpr int S0 = W <= 3 ? 3 : (W <= 5 ? W : (W <= 8 ? 8 : 11));
+    constexpr int S1 = W == 3 ? 4 : (W == 4 ? 5 : (W == 5 ? 8 : 0));  // 0: linear
+    if (a.m <= stripe_limit<S0>()) return launch_filter_variant<W, 3, S0>(a, stream);
+    if constexpr (32 * W <= stripe_limit<S0>())
+      return cudaErrorInvalidValue;
+    else
+      return launch_filter_variant<W, 3, S1>(a, stream);
   }
 }
 

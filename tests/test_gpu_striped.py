@@ -1,0 +1,42 @@
+"""Bit-exact parity of the striped kernels with the CPU oracle at the read
+lengths where the number of stripes changes and where the last row is full,
+nearly full or just begun (integer work, tolerance 0)."""
+import numpy as np
+import pytest
+import torch
+
+from oracle import oracle as O
+from paper_2103_14978_gb300 import device_data as dd, gk
+from tests.gpu_helpers import GpuRun, assert_same, oracle_run, require_gpu, small_workload
+
+pytestmark = pytest.mark.gpu
+
+EDGES = [33, 63, 64, 65, 91, 92, 93, 96, 97, 100, 101, 125, 126, 127, 128, 129, 150, 155, 156, 157, 160, 161, 192,
+         224, 248, 253, 254, 255, 256, 257, 300, 319, 320, 321]
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _gpu():
+    require_gpu()
+
+
+@pytest.mark.parametrize("m", EDGES)
+def test_sweep_at_stripe_edges(m):
+    """Neighbouring pairs that share a read (an odd pair count, so that the
+    last one is alone) and pairs in random order; both counts; a genome with
+    few and with many N (one thread per pair, the queue of defined pairs)."""
+    for cands, n_frac, mode in ((4, 0.0, gk.GK_COUNT_RUNS4), (5, 0.0, gk.GK_COUNT_POPCOUNT),
+                                (1, 0.0, gk.GK_COUNT_RUNS4), (6, 0.002, gk.GK_COUNT_RUNS4)):
+        w = small_workload(m, 1501, seed=3000 + m + cands, n_frac=n_frac, read_n_frac=n_frac, cands=cands)
+        if cands == 5:
+            perm = np.random.default_rng(m).permutation(w.n_pairs)
+            w.pair_read, w.pair_off = w.pair_read[perm].copy(), w.pair_off[perm].copy()
+        run = GpuRun(w)
+        r = run.reads
+        acc, ed = gk.gk_filter_sweep(run.ref, r.packed, r.stride_words, r.n_reads, r.nflag, m, run.pairs.pair_read,
+                                     run.pairs.pair_off, 0, 30, count_mode=mode)
+        torch.cuda.synchronize()
+        for e in range(31):
+            assert_same((acc[e].cpu().numpy(), dd.edits_u16(ed[e])),
+                        oracle_run(w, e, O.RUNS4 if mode == gk.GK_COUNT_RUNS4 else O.POPCOUNT),
+                        f"m={m} cands={cands} e={e}")
