@@ -783,20 +783,24 @@ template <int W, int S>
 __device__ __forceinline__ void sweep_and_write(const FilterArgs &a, uint64_t p, const PairData<W> &x) {
   const uint32_t e_lo = a.fixed_e, e_hi = a.sweep_hi, kmax = x.m - 1;
   const uint32_t Klo = min(e_lo, kmax), Khi = min(e_hi, kmax);
-  // The common case (K in e_lo..e_hi, below m-1) writes one row: its
-  // pointers advance by a row per shift count.
+  // The rows come in order, one per K and, at K = m-1, all that are left:
+  // their pointers advance by a row each.
   uint8_t *acc_row = a.accept + p;
   uint16_t *ed_row = a.edits + p;
   auto emit = [&](uint32_t K, const uint32_t (&c)[1]) {
-    if (!a.result_byte && K >= e_lo && K < kmax) {
-      *acc_row = c[0] <= K;
-      *ed_row = (uint16_t)c[0];
+    const uint32_t last = K == kmax ? e_hi : K;
+    uint32_t e = max(K, e_lo);
+#pragma unroll 1
+    do {
+      if (a.result_byte) {
+        *acc_row = (uint8_t)min(c[0], GK_RESULT_MAX_COUNT);
+      } else {
+        *acc_row = c[0] <= e;
+        *ed_row = (uint16_t)c[0];
+      }
       acc_row += a.out_stride;
       ed_row += a.out_stride;
-      return;
-    }
-    const uint32_t first = K > e_lo ? K : e_lo, last = K == kmax ? e_hi : K;
-    for (uint32_t e = first; e <= last; ++e) write_count(a, p + (uint64_t)(e - e_lo) * a.out_stride, c[0], e);
+    } while (++e <= last);
   };
   if constexpr (S > 0) {
     uint32_t rh[S], rl[S], gh[1][S], gl[1][S];
@@ -1005,7 +1009,9 @@ __global__ void __launch_bounds__(kFilterThreads, MinBlocks<W, COMPACT, S>::valu
       qn += __popc(need);
       __syncwarp();
     }
-    while (qn >= 32 || (!more && qn > 0)) {
+    // One place filters, the drain included: the code of a second one would
+    // not fit the instruction cache beside it.
+    while (qn >= 32 || (!more && (qn > 0 || pend >= 0))) {
       const uint32_t take = qn < 32 ? qn : 32;
       const bool has = (uint32_t)lane < take;
       const int nb = pend == 0 ? 1 : 0;
@@ -1033,17 +1039,13 @@ __global__ void __launch_bounds__(kFilterThreads, MinBlocks<W, COMPACT, S>::valu
         cp_async_wait<1>();  // the previous batch's copies have landed
         filter_staged();
       }
-      pend = nb;
+      pend = take > 0 ? nb : -1;
       pend_has = has;
       pend_p = np;
       pend_off = noff;
       pend_e = ne;
     }
     if (!more) break;
-  }
-  if (pend >= 0) {
-    cp_async_wait<0>();
-    filter_staged();
   }
 }
 
@@ -1149,38 +1151,32 @@ __global__ void __launch_bounds__(kFilterThreads, S == 5 ? 3 : 4) sweep_pair2_ke
     // rows keep that alignment.
     const bool pack = (((uintptr_t)a.accept | (a.result_byte ? 0u : (uintptr_t)a.edits)) & 3u) == 0 &&
                       (a.out_stride & 1u) == 0;
-    const bool one_row = pack && !a.result_byte;
-    // The common case (K in e_lo..e_hi, below m-1) writes one row.
     uint8_t *acc_row = a.accept + base;
     uint16_t *ed_row = a.edits + base;
-    auto emit = [&](uint32_t K, const uint32_t (&c)[2]) {
-      if (one_row && K < kmax) {
-        *reinterpret_cast<uint32_t *>(ed_row + lo) = c[0] | (c[1] << 16);
-        *reinterpret_cast<uint16_t *>(acc_row + lo) =
-            (uint16_t)((c[0] <= K ? 1u : 0u) | (c[1] <= K ? 0x100u : 0u));
+    auto emit = [&](uint32_t K, const uint32_t (&c)[2]) {  // rows in order, as in sweep_and_write
+      const uint32_t last = K == kmax ? e_hi : K;
+      uint32_t e = max(K, e_lo);
+#pragma unroll 1
+      do {
+        uint32_t b0 = c[0] <= e ? 1u : 0u, b1 = c[1] <= e ? 1u : 0u;
+        if (a.result_byte) {
+          b0 = min(c[0], GK_RESULT_MAX_COUNT);
+          b1 = min(c[1], GK_RESULT_MAX_COUNT);
+        } else if (pack) {
+          *reinterpret_cast<uint32_t *>(ed_row + lo) = c[0] | (c[1] << 16);
+        } else {
+          ed_row[lo] = (uint16_t)c[0];
+          ed_row[lo + 1] = (uint16_t)c[1];
+        }
+        if (pack) {
+          *reinterpret_cast<uint16_t *>(acc_row + lo) = (uint16_t)(b0 | (b1 << 8));
+        } else {
+          acc_row[lo] = (uint8_t)b0;
+          acc_row[lo + 1] = (uint8_t)b1;
+        }
         acc_row += a.out_stride;
         ed_row += a.out_stride;
-        return;
-      }
-      const uint32_t first = K > e_lo ? K : e_lo, last = K == kmax ? e_hi : K;
-      for (uint32_t e = first; e <= last; ++e) {
-        const uint64_t o = (uint64_t)(e - e_lo) * a.out_stride;
-        if (pack) {
-          uint32_t b0, b1;
-          if (a.result_byte) {
-            b0 = min(c[0], GK_RESULT_MAX_COUNT);
-            b1 = min(c[1], GK_RESULT_MAX_COUNT);
-          } else {
-            b0 = c[0] <= e;
-            b1 = c[1] <= e;
-            *reinterpret_cast<uint32_t *>(a.edits + o + p0) = c[0] | (c[1] << 16);
-          }
-          *reinterpret_cast<uint16_t *>(a.accept + o + p0) = (uint16_t)(b0 | (b1 << 8));
-        } else {
-          write_count(a, p0 + o, c[0], e);
-          write_count(a, p1 + o, c[1], e);
-        }
-      }
+      } while (++e <= last);
     };
     if constexpr (S > 0) {
       uint32_t rh[S], rl[S], gh[2][S], gl[2][S];
