@@ -37,7 +37,15 @@
 
 namespace gk {
 
-constexpr int kFilterThreads = 256;
+// Threads per block.  A block's warps load together and its registers are
+// freed together, so smaller blocks interleave one block's loads with
+// another's arithmetic: against 256 threads (same registers, GB300) 150 bp at
+// e = 3 ran 0.248 -> 0.213 ms, 250 bp at e = 5 0.324 -> 0.259, 100 bp at e = 5
+// 0.461 -> 0.434; 64 threads the same as 128.
+constexpr int kFilterThreads = 128;
+// The persistent warps of the queue of defined pairs already interleave
+// (128 threads measured 1% slower).
+constexpr int kQueueThreads = 256;
 
 template <int W>
 __device__ __forceinline__ void amend_and(const uint32_t (&d)[W], uint32_t (&acc)[W],
@@ -723,9 +731,9 @@ __device__ __forceinline__ uint32_t filter_loaded_deferred(const FilterArgs &a, 
 template <int W, bool COMPACT, int S = 0>
 struct MinBlocks {
   static constexpr int value =
-      S > 0 ? (S <= 4 ? 4 : (S == 5 ? 3 : 2))
+      S > 0 ? (COMPACT ? 1 : 2) * (S <= 4 ? 4 : (S == 5 ? 3 : 2))
       : COMPACT ? (W <= 2 ? 5 : (W <= 4 ? 4 : (W <= 6 ? 3 : (W <= 8 ? 2 : 1))))
-              : (W <= 2 ? 6 : (W <= 4 ? 5 : (W == 5 ? 4 : (W == 6 ? 3 : (W <= 8 ? 2 : 1)))));
+              : (W <= 2 ? 12 : (W <= 4 ? 10 : (W == 5 ? 8 : (W == 6 ? 6 : (W <= 8 ? 4 : 2)))));
 };
 
 // Status of a loaded pair: 0 filter, 1 undefined (N in read or window),
@@ -887,7 +895,7 @@ __device__ __forceinline__ void cp_async_wait() {
   asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory");
 }
 
-constexpr int kFilterWarps = kFilterThreads / 32;
+constexpr int kFilterWarps = kFilterThreads / 32, kQueueWarps = kQueueThreads / 32;
 
 // Words of one staged batch (32 pairs): W read words and W + 1 window words
 // per pair, stored word-major ([word][lane]) so that lanes touch consecutive
@@ -896,7 +904,7 @@ template <int W>
 constexpr int kStageWords = (2 * W + 1) * 32;
 template <int W>
 constexpr size_t compact_smem_bytes() {
-  return (size_t)kFilterWarps * 2 * kStageWords<W> * sizeof(uint2);
+  return (size_t)kQueueWarps * 2 * kStageWords<W> * sizeof(uint2);
 }
 
 // VARIANT 0: any thresholds; 1: every shift count of the launch is < 32;
@@ -914,7 +922,8 @@ constexpr size_t compact_smem_bytes() {
 // behind the arithmetic of the other.  Dynamic shared memory:
 // compact_smem_bytes<W>().
 template <int W, int VARIANT, bool COMPACT, int S = 0>
-__global__ void __launch_bounds__(kFilterThreads, MinBlocks<W, COMPACT, S>::value) filter_kernel(const FilterArgs a) {
+__global__ void __launch_bounds__(COMPACT ? kQueueThreads : kFilterThreads, MinBlocks<W, COMPACT, S>::value)
+    filter_kernel(const FilterArgs a) {
   if (!COMPACT) {
     const uint64_t p = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x;
     const bool active = p < a.n_pairs;
@@ -935,12 +944,12 @@ __global__ void __launch_bounds__(kFilterThreads, MinBlocks<W, COMPACT, S>::valu
     return;
   }
   extern __shared__ uint2 stage_all[];
-  __shared__ uint32_t q_p[kFilterWarps][64], q_rid[kFilterWarps][64], q_off[kFilterWarps][64];
+  __shared__ uint32_t q_p[kQueueWarps][64], q_rid[kQueueWarps][64], q_off[kQueueWarps][64];
   const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
   uint2 *stage = stage_all + wib * 2 * kStageWords<W>;
   const uint64_t n_chunks = (a.n_pairs + 31) / 32;
-  const uint64_t n_warps = (uint64_t)gridDim.x * kFilterWarps;
-  uint64_t c = blockIdx.x * (uint64_t)kFilterWarps + wib;
+  const uint64_t n_warps = (uint64_t)gridDim.x * kQueueWarps;
+  uint64_t c = blockIdx.x * (uint64_t)kQueueWarps + wib;
   // Load pipeline over this warp's chunks.  Wide reads (W >= 7, registers to
   // spare) run it two deep: while the warp classifies chunk c and filters,
   // the N information of its next chunk and the ids of the chunk after are
@@ -1060,7 +1069,7 @@ constexpr bool kPair2Wide = false;
 // 57.5 Gpairs/s; the sweep 1.307 -> 1.280 ms), the same at e = 0.
 template <int W>
 struct MinBlocks2 {
-  static constexpr int value = 4;
+  static constexpr int value = 8;
 };
 
 // Deferred erosion (VARIANT 2), two pairs per thread: pairs 2t and 2t+1.  When both are filtered and share their read
@@ -1126,7 +1135,7 @@ __global__ void __launch_bounds__(kFilterThreads, MinBlocks2<W>::value) filter_p
 // 4 (3 blocks measured 1% slower at 100 bp), 80 S = 5 (2 blocks 7% slower at
 // 150 bp; one pair per thread 12% slower).
 template <int W, int S>
-__global__ void __launch_bounds__(kFilterThreads, S == 5 ? 3 : 4) sweep_pair2_kernel(const FilterArgs a) {
+__global__ void __launch_bounds__(kFilterThreads, S == 5 ? 6 : 8) sweep_pair2_kernel(const FilterArgs a) {
   const uint64_t base = blockIdx.x * (uint64_t)(2 * kFilterThreads);
   const uint32_t lo = 2 * threadIdx.x;
   const uint64_t p0 = base + lo, p1 = p0 + 1;
@@ -1265,15 +1274,16 @@ cudaError_t launch_filter_variant(const FilterArgs &a, cudaStream_t stream) {
     err = cudaDeviceGetAttribute(&count, cudaDevAttrMultiProcessorCount, dev);
     if (err != cudaSuccess) return err;
     int n = 0;
-    err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, filter_kernel<W, VARIANT, true, S>, kFilterThreads, smem);
+    err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, filter_kernel<W, VARIANT, true, S>, kQueueThreads, smem);
     if (err != cudaSuccess) return err;
     blocks_per_sm = n < 1 ? 1 : n;
     sms[dev].store(count, std::memory_order_relaxed);
     per_sm[dev].store(blocks_per_sm, std::memory_order_release);
   }
+  blocks = (unsigned)((a.n_pairs + kQueueThreads - 1) / kQueueThreads);
   const uint64_t wave = 4ull * (uint64_t)sms[dev].load(std::memory_order_relaxed) * (uint64_t)blocks_per_sm;
   if (blocks > wave) blocks = (unsigned)wave;
-  filter_kernel<W, VARIANT, true, S><<<blocks, kFilterThreads, smem, stream>>>(a);
+  filter_kernel<W, VARIANT, true, S><<<blocks, kQueueThreads, smem, stream>>>(a);
   return cudaGetLastError();
   }
 }

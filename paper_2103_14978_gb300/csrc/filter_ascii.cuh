@@ -49,7 +49,7 @@ __device__ __forceinline__ void load_word_bytes(const uint8_t *row, uint32_t w, 
 // would spill with the encoder's registers.
 template <int W>
 struct MinBlocksAscii {
-  static constexpr int value = W <= 2 ? 5 : (W <= 4 ? 4 : MinBlocks<W, false>::value);
+  static constexpr int value = W <= 2 ? 10 : (W <= 4 ? 8 : MinBlocks<W, false>::value);
 };
 
 template <int W, int VARIANT>

@@ -53,6 +53,25 @@ __host__ __device__ __forceinline__ uint32_t st_popc(uint32_t x) {
 #endif
 }
 
+__host__ __device__ __forceinline__ uint32_t st_brev(uint32_t x) {
+#ifdef __CUDA_ARCH__
+  return __brev(x);
+#else
+  uint32_t r = 0;
+  for (int i = 0; i < 32; ++i) r |= ((x >> i) & 1u) << (31 - i);
+  return r;
+#endif
+}
+
+// The low 32 bits of hi:lo >> s, s in 0..32.
+__host__ __device__ __forceinline__ uint32_t st_shr64(uint32_t lo, uint32_t hi, uint32_t s) {
+#ifdef __CUDA_ARCH__
+  return __funnelshift_rc(lo, hi, s);
+#else
+  return (uint32_t)((((uint64_t)hi << 32) | lo) >> s);
+#endif
+}
+
 // The 3-input logic function with truth table LUT (a = 0xF0, b = 0xCC, c =
 // 0xAA).
 template <uint32_t LUT>
@@ -365,6 +384,130 @@ __host__ __device__ __forceinline__ void striped_exact(uint32_t m, uint32_t Klo,
     }
     v0 = v1;
     v1 = v2;
+  }
+}
+
+// Corrections next to the vacated runs of one shift count K <= 30 (the
+// deferred erosion of filter.cuh, deferred_counts), from the linear planes:
+// lo, bit p: position p <= K + 1; hi, bit b: position m - 32 + b.  1s are
+// positions the final vector loses.
+template <int W>
+__host__ __device__ __forceinline__ void end_corrections(uint32_t m, uint32_t K, const uint32_t (&rh)[W],
+                                                         const uint32_t (&rl)[W], const uint32_t (&gh)[W],
+                                                         const uint32_t (&gl)[W], uint32_t &lo, uint32_t &hi) {
+  static_assert(W >= 2, "more than one word");
+  const uint32_t r1k = (2u << K) - 2u;  // bits 1..K
+  auto terms = [&](uint32_t h, uint32_t l, uint32_t h0, uint32_t l0, uint32_t h1, uint32_t l1) -> uint32_t {
+    // h, l: window bases from the end inwards; h0 .. l1: the read's end base and the next, broadcast
+    const uint32_t a0 = (h ^ h0) | (l ^ l0), a1 = (h ^ h1) | (l ^ l1), vac = h | l;
+    const uint32_t c2 = (vac << 1) | a0 | (a1 >> 1), c1 = (vac << 2) | (vac << 1) | a0;
+    return (~(c1 & c2) & r1k) | ((~c2 & r1k) << 1);
+  };
+  const uint32_t tail = m - 32u * (W - 1);  // 1..32
+  lo = terms(gh[0], gl[0], 0u - (rh[0] & 1u), 0u - (rl[0] & 1u), 0u - ((rh[0] >> 1) & 1u), 0u - ((rl[0] >> 1) & 1u));
+  const uint32_t xh = st_shr64(rh[W - 2], rh[W - 1], tail), xl = st_shr64(rl[W - 2], rl[W - 1], tail);  // last 32
+  hi = st_brev(terms(st_brev(st_shr64(gh[W - 2], gh[W - 1], tail)), st_brev(st_shr64(gl[W - 2], gl[W - 1], tail)),
+                     0u - (xh >> 31), 0u - (xl >> 31), 0u - ((xh >> 30) & 1u), 0u - ((xl >> 30) & 1u)));
+}
+
+// The count at one shift count K (1 <= K <= 30, K < m) of NP pairs that share
+// one read: deferred erosion (filter.cuh, deferred_counts) on stripes.  The
+// loop ANDs dilations with the vacated positions set before them and the AND
+// is eroded once; clo, chi are the pairs' end_corrections.  A step takes 8 S
+// logic ops, 2 S fewer than an exact one; the corrections and their striping
+// cost about 4 (S = 4) or 3 (S = 8) steps' worth of that.
+template <int W, int S, int NP, bool WHOLE>
+__host__ __device__ __forceinline__ void striped_deferred(uint32_t m, uint32_t K, int count_mode,
+                                                          const uint32_t (&rh)[S], const uint32_t (&rl)[S],
+                                                          const uint32_t (&gh)[NP][S], const uint32_t (&gl)[NP][S],
+                                                          const uint32_t (&clo)[NP], const uint32_t (&chi)[NP],
+                                                          uint32_t (&count)[NP]) {
+  uint32_t acc[NP][S];  // position p at index p + 1
+#pragma unroll
+  for (int j = 0; j < NP; ++j) {
+    uint32_t d[S];
+#pragma unroll
+    for (int w = 0; w < S; ++w) d[w] = lop3<0xF6>(rh[w] ^ gh[j][w], rl[w], gl[j][w]);
+    stripe_or3<S>(d, acc[j]);
+  }
+  // As in striped_exact, in positions: u: those of the -k copy that hold a
+  // read base; v0, v1: the rows vacated in the +k mask.
+  uint32_t ph[S], pl[S], nh[S], nl[S], lm[S], u[S];
+  stripe_masks<W, S>(m, lm);
+#pragma unroll
+  for (int w = 0; w < S; ++w) {
+    ph[w] = nh[w] = rh[w];
+    pl[w] = nl[w] = rl[w];
+    u[w] = lm[w];
+  }
+  // S odd: what rotates in at the top of u would be a read base past m.
+  constexpr uint32_t kKeep = (S & 1) ? ~row_bit<S>(31) : 0xffffffffu;
+  uint32_t v0 = 0u;
+  for (uint32_t kb = 0; kb < K; kb += S) {
+    const uint32_t v1 = row_up<S>(v0) | 1u;
+#pragma unroll
+    for (int t = 0; t < S; ++t) {  // k = kb + t + 1
+      if (kb + (uint32_t)t + 1u > K) break;
+      constexpr int kS = S;
+      const int up = (kS - 1 - t) % kS;
+      ph[up] = row_up<S>(ph[up]);
+      pl[up] = row_up<S>(pl[up]);
+      if (WHOLE) {
+        ph[up] &= lm[0];
+        pl[up] &= lm[0];
+      }
+      nh[t] = row_down<S>(nh[t]);
+      nl[t] = row_down<S>(nl[t]);
+      u[t] = row_down<S>(u[t]) & kKeep;
+#pragma unroll
+      for (int j = 0; j < NP; ++j) {
+        uint32_t d[S], x[S], y[S];
+#pragma unroll
+        for (int w = 0; w < S; ++w) {  // +k
+          const int i = (w + kS - 1 - t) % kS;
+          const uint32_t v = w <= t ? v1 : v0;
+          if (WHOLE)
+            d[w] = lop3<0xF6>(lop3<0xDE>(ph[i], v, gh[j][w]), pl[i], gl[j][w]);
+          else
+            d[w] = lop3<0xEA>(lop3<0xF6>(ph[i] ^ gh[j][w], pl[i], gl[j][w]), lm[w], v);
+        }
+        stripe_or3<S>(d, x);
+#pragma unroll
+        for (int w = 0; w < S; ++w) {  // -k
+          const int i = (w + t + 1) % kS;
+          d[w] = lop3<0xF6>(lop3<0x7B>(nh[i], u[i], gh[j][w]), nl[i], gl[j][w]);
+        }
+        if (S & 1) {  // positions past m, all vacated, must not come round to position 0
+          d[S - 1] &= ~row_bit<S>(31);
+          d[S - 2] &= ~row_bit<S>(31);
+        }
+        stripe_or3<S>(d, y);
+#pragma unroll
+        for (int w = 0; w < S; ++w) acc[j][w] = lop3<0x80>(acc[j][w], x[w], y[w]);
+      }
+    }
+    v0 = v1;
+  }
+  // hi's bit b is index m - 30 + b of the final vector (position + 2).
+  const uint32_t tail = m - 32u * (W - 1), sh = (tail + 2u) & 31u;
+  const bool top = tail >= 30;
+#pragma unroll
+  for (int j = 0; j < NP; ++j) {
+    constexpr int kC = W < S ? W + 1 : W;
+    uint32_t c[kC], cs[S], f[S];
+#pragma unroll
+    for (int w = 0; w < kC; ++w) c[w] = 0u;
+    c[0] = clo[j] << 2;
+    c[1] |= clo[j] >> 30;
+    const uint32_t l = chi[j] << sh, h = st_shr64(chi[j], 0u, 32u - sh);
+    c[W - 2] |= top ? 0u : l;
+    c[W - 1] |= top ? l : h;
+    if (W < S) c[W < S ? W : 0] |= top ? h : 0u;
+    stripe_linear<kC, S>(c, cs);
+    stripe_and3<S>(acc[j], f);
+#pragma unroll
+    for (int w = 0; w < S; ++w) f[w] &= ~cs[w];
+    count[j] = stripe_count<S>(f, count_mode);
   }
 }
 
