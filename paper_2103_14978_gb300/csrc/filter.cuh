@@ -170,7 +170,7 @@ __device__ __forceinline__ void load_pair(const FilterArgs &a, uint64_t p, PairD
   x.off = a.pair_off[p];
   x.e = a.pair_e ? (uint32_t)a.pair_e[p] : a.fixed_e;
   x.m = a.m;
-  x.status = ((uint64_t)x.rid >= a.n_reads || (uint64_t)x.off + a.m > a.ref_len) ? 2 : 0;
+  x.status = (x.rid > a.rid_last || x.off >= a.off_end) ? 2 : 0;
   x.nflag = 0;
   x.ni = make_uint2(0, 0xffffffffu);
   if (x.status == 0 && a.m > 0) {
@@ -712,6 +712,38 @@ __device__ __forceinline__ void striped_read(const PairData<W> &x, uint32_t (&rh
   stripe_linear<W, S>(l, rl);
 }
 
+// Counts at one shift count K (1 .. 30, below m) of NP pairs that share one
+// read (x0's), striped with deferred erosion.
+template <int W, int S, int NP, bool WHOLE>
+__device__ __forceinline__ void striped_counts(const PairData<W> &x0, const PairData<W> &x1, uint32_t m, uint32_t K,
+                                               int count_mode, uint32_t (&count)[NP]) {
+  uint32_t rh[S], rl[S], gh[NP][S], gl[NP][S], h[W], l[W], wh[W], wl[W], lo[NP], hi[NP];
+  read_planes<W>(x0, h, l);
+  stripe_linear<W, S>(h, rh);
+  stripe_linear<W, S>(l, rl);
+#pragma unroll
+  for (int j = 0; j < NP; ++j) {
+    window_planes<W>(j ? x1 : x0, wh, wl);
+    end_corrections<W>(m, K, h, l, wh, wl, lo[j], hi[j]);
+    stripe_linear<W, S>(wh, gh[j]);
+    stripe_linear<W, S>(wl, gl[j]);
+  }
+  striped_deferred<W, S, NP, WHOLE>(m, K, count_mode, rh, rl, gh, gl, lo, hi, count);
+}
+
+// One pair's count at the launch's one length and shift count, striped
+// (uniform values: the masks stay in scalar registers).
+template <int W, int S>
+__device__ __forceinline__ uint32_t filter_loaded_striped(const FilterArgs &a, const PairData<W> &x) {
+  const uint32_t K = min(a.fixed_e, a.m - 1);
+  uint32_t c[1];
+  if (a.m % S == 0)
+    striped_counts<W, S, 1, true>(x, x, a.m, K, a.count_mode, c);
+  else
+    striped_counts<W, S, 1, false>(x, x, a.m, K, a.count_mode, c);
+  return c[0];
+}
+
 template <int W, bool DIRECT = false>
 __device__ __forceinline__ uint32_t filter_loaded_deferred(const FilterArgs &a, const PairData<W> &x) {
   uint32_t rh[W], rl[W], gh[1][W], gl[1][W], count[1];
@@ -742,12 +774,11 @@ template <int W>
 __device__ __forceinline__ int pair_status(const FilterArgs &a, const PairData<W> &x) {
   int status = x.status;
   if (status == 0 && a.m > 0) {
-    if (x.nflag) {
-      status = 1;
-    } else {
+    if (x.nflag) status = 1;
+    if (a.ref_nidx) {  // a valid pair's window ends below 2^32
       const uint32_t q = x.ni.x >> (x.off & 31);
-      const uint64_t first = q ? (uint64_t)x.off + (uint32_t)(__ffs(q) - 1) : (uint64_t)x.ni.y;
-      if (first < (uint64_t)x.off + a.m) status = 1;
+      const uint32_t first = q ? x.off + (uint32_t)(__ffs(q) - 1) : x.ni.y;
+      if (first < x.off + a.m) status = 1;
     }
   }
   return status;
@@ -830,9 +861,13 @@ __device__ __forceinline__ void filter_and_write(const FilterArgs &a, uint64_t p
   if constexpr (VARIANT == 3) {
     sweep_and_write<W, S>(a, p, x);
   } else {
-    const uint32_t count = VARIANT == 4   ? filter_loaded_deferred<W, true>(a, x)
-                           : VARIANT == 2 ? filter_loaded_deferred<W>(a, x)
-                                          : filter_loaded<W, VARIANT == 1>(a, x);
+    uint32_t count;
+    if constexpr (S > 0)
+      count = filter_loaded_striped<W, S>(a, x);
+    else
+      count = VARIANT == 4   ? filter_loaded_deferred<W, true>(a, x)
+              : VARIANT == 2 ? filter_loaded_deferred<W>(a, x)
+                             : filter_loaded<W, VARIANT == 1>(a, x);
     write_count(a, p, count, x.e);
   }
 }
@@ -852,7 +887,7 @@ __device__ __forceinline__ void chunk_issue(const FilterArgs &a, ChunkLoads &x) 
   x.nflag = 0;
   x.ni = make_uint2(0u, 0xffffffffu);
   if (x.state < 0) return;
-  if ((uint64_t)x.rid >= a.n_reads || (uint64_t)x.off + a.m > a.ref_len) {
+  if (x.rid > a.rid_last || x.off >= a.off_end) {
     x.state = 2;
   } else if (a.m == 0) {
     x.state = 3;
@@ -868,8 +903,8 @@ __device__ __forceinline__ int chunk_status(const FilterArgs &a, const ChunkLoad
   if (x.state != 0) return x.state;
   if (x.nflag) return 1;
   const uint32_t q = x.ni.x >> (x.off & 31);
-  const uint64_t first = q ? (uint64_t)x.off + (uint32_t)(__ffs(q) - 1) : (uint64_t)x.ni.y;
-  return first < (uint64_t)x.off + a.m ? 1 : 0;
+  const uint32_t first = q ? x.off + (uint32_t)(__ffs(q) - 1) : x.ni.y;
+  return first < x.off + a.m ? 1 : 0;
 }
 
 __device__ __forceinline__ void chunk_ids(const FilterArgs &a, uint64_t c, uint64_t n_chunks, int lane,
@@ -909,8 +944,8 @@ constexpr size_t compact_smem_bytes() {
 
 // VARIANT 0: any thresholds; 1: every shift count of the launch is < 32;
 // 2: edge OR on and one threshold in 2..30, deferred erosion; 3: edge OR on,
-// a sweep of thresholds up to 30 (sweep_and_write; striped in S words or, S =
-// 0, linear).
+// a sweep of thresholds up to 30 (sweep_and_write).  2 and 3 are striped in S
+// words or, S = 0, linear.
 //
 // COMPACT false: one thread per pair.  COMPACT true (inputs with many
 // undefined pairs): persistent warps take 32 pairs at a time (their ids
@@ -1079,8 +1114,12 @@ struct MinBlocks2 {
 // is filtered on its own.  VARIANT 4: one threshold whose shift count KC
 // (0..2, below m) is a compile-time constant, so the shift steps unroll and
 // the end corrections of K = 0 vanish.
-template <int W, int VARIANT, int KC = -1>
-__global__ void __launch_bounds__(kFilterThreads, MinBlocks2<W>::value) filter_pair2_kernel(const FilterArgs a) {
+//
+// S > 0: striped; of pairs that do not share a read the second is then loaded
+// anew, as in the sweep.
+template <int W, int VARIANT, int KC = -1, int S = 0>
+__global__ void __launch_bounds__(kFilterThreads, S == 5 ? 6 : MinBlocks2<W>::value)
+    filter_pair2_kernel(const FilterArgs a) {
   const uint64_t t = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x;
   const uint64_t p0 = 2 * t, p1 = p0 + 1;
   const bool act0 = p0 < a.n_pairs, act1 = p1 < a.n_pairs;
@@ -1103,11 +1142,19 @@ __global__ void __launch_bounds__(kFilterThreads, MinBlocks2<W>::value) filter_p
   if (s0 > 0) write_trivial(a, p0, s0);
   if (s1 > 0) write_trivial(a, p1, s1);
   if (s0 == 0 && s1 == 0 && x0.rid == x1.rid) {
-    uint32_t rh[W], rl[W], gh[2][W], gl[2][W], count[2];
-    pair_planes<W>(x0, rh, rl, gh[0], gl[0]);
-    window_planes<W>(x1, gh[1], gl[1]);
     const uint32_t K = KC >= 0 ? (uint32_t)KC : min(a.fixed_e, a.m - 1);
-    deferred_counts<W, 2, (KC >= 0)>(a, a.m, K, rh, rl, gh, gl, count);
+    uint32_t count[2];
+    if constexpr (S > 0) {
+      if (a.m % S == 0)
+        striped_counts<W, S, 2, true>(x0, x1, a.m, K, a.count_mode, count);
+      else
+        striped_counts<W, S, 2, false>(x0, x1, a.m, K, a.count_mode, count);
+    } else {
+      uint32_t rh[W], rl[W], gh[2][W], gl[2][W];
+      pair_planes<W>(x0, rh, rl, gh[0], gl[0]);
+      window_planes<W>(x1, gh[1], gl[1]);
+      deferred_counts<W, 2, (KC >= 0)>(a, a.m, K, rh, rl, gh, gl, count);
+    }
     // The two pairs are adjacent: one 2-byte accept store and one 4-byte
     // count store when the buffers allow it.
     if (!a.result_byte && ((uintptr_t)a.accept & 1u) == 0 && ((uintptr_t)a.edits & 3u) == 0) {
@@ -1119,6 +1166,13 @@ __global__ void __launch_bounds__(kFilterThreads, MinBlocks2<W>::value) filter_p
       write_count(a, p0, count[0], a.fixed_e);
       write_count(a, p1, count[1], a.fixed_e);
     }
+  } else if constexpr (S > 0) {
+#pragma unroll 1
+    for (int j = 0; j < 2; ++j) {
+      if ((j ? s1 : s0) != 0) continue;
+      if (j) load_pair<W>(a, p1, x0);
+      filter_and_write<W, VARIANT, S>(a, p0 + j, x0);
+    }
   } else {
     if (s0 == 0) filter_and_write<W, VARIANT>(a, p0, x0);
     if (s1 == 0) filter_and_write<W, VARIANT>(a, p1, x1);
@@ -1129,8 +1183,9 @@ __global__ void __launch_bounds__(kFilterThreads, MinBlocks2<W>::value) filter_p
 // filtered and share their read, its shifted copies and their masks serve both
 // windows, and each threshold's two results go out as one 2-byte and one
 // 4-byte store.  Rows are addressed as a block's base plus a 32-bit offset, so
-// that their advance is scalar work.  Pairs that do not share are loaded anew,
-// one after the other (keeping both over the shared form's registers spills).
+// that their advance is scalar work.  Of pairs that do not share a read the
+// second is loaded anew (keeping both beside the shared form's registers
+// spills).
 // S: stripes, or 0 for the linear form.  Blocks per SM: 64 registers hold S <=
 // 4 (3 blocks measured 1% slower at 100 bp), 80 S = 5 (2 blocks 7% slower at
 // 150 bp; one pair per thread 12% slower).
@@ -1206,7 +1261,7 @@ __global__ void __launch_bounds__(kFilterThreads, S == 5 ? 6 : 8) sweep_pair2_ke
 #pragma unroll 1
     for (int j = 0; j < 2; ++j) {
       if ((j ? s1 : s0) != 0) continue;
-      load_pair<W>(a, p0 + j, x0);
+      if (j) load_pair<W>(a, p1, x0);
       sweep_and_write<W, S>(a, p0 + j, x0);
     }
   }
@@ -1228,7 +1283,7 @@ cudaError_t launch_filter_variant(const FilterArgs &a, cudaStream_t stream) {
         return cudaGetLastError();
       }
     }
-    if constexpr ((VARIANT == 2 || VARIANT == 4) && W <= 4) {
+    if constexpr ((VARIANT == 2 || VARIANT == 4) && (W <= 4 || S == 5)) {
       if (a.m > 0) {
         if constexpr (VARIANT == 4) {
           // shift count = the threshold, 0..2, below m (checked by the caller)
@@ -1239,7 +1294,7 @@ cudaError_t launch_filter_variant(const FilterArgs &a, cudaStream_t stream) {
             default: return cudaErrorInvalidValue;
           }
         } else {
-          filter_pair2_kernel<W, VARIANT><<<grid, kFilterThreads, 0, stream>>>(a);
+          filter_pair2_kernel<W, VARIANT, -1, S><<<grid, kFilterThreads, 0, stream>>>(a);
         }
         return cudaGetLastError();
       }
@@ -1307,6 +1362,29 @@ cudaError_t launch_sweep(const FilterArgs &a, cudaStream_t stream) {
     else
       return launch_filter_variant<W, 3, S1>(a, stream);
   }
+}
+
+// Launches VARIANT 2 (one threshold, shift count 2 .. 30, edge OR on) over
+// reads of W words: striped from the shift count at which it wins, also where
+// neighbouring pairs name different reads (they cost it a second load).
+// Striping a read and a window takes as long as about three shift steps, and
+// rows are partly empty at m well below 32 S.  Measured on GB300, launches
+// alone, linear / striped in us, pairs in fours of one read: 8M pairs of 76 bp
+// K = 4 144 / 135 (every pair its own read: 168 / 187), K = 8 211 / 186 (248 /
+// 236); 10M of 100 bp K = 5 232 / 232, 7 289 / 257, 10 375 / 302 (455 / 407); 6M
+// of 150 bp K = 5 197 / 158, 8 266 / 193 (267 / 263), 15 441 / 285; 5M of 170 bp
+// K = 9 279 / 315, 17 477 / 451; of 200 bp K = 7 258 / 267, 10 340 / 311; 4M of
+// 250 bp K = 5 188 / 209, 8 257 / 242, 25 687 / 473; 3M of 280 bp K = 14 345 /
+// 326; of 300 bp K = 9 258 / 258, 15 400 / 347; 128 and 160 bp (S = 5 and 8 with
+// 20 rows) no faster up to K = 16.
+template <int W>
+cudaError_t launch_single(const FilterArgs &a, cudaStream_t stream) {
+  if constexpr (W >= 3 && W <= 10) {
+    constexpr int S = W <= 5 ? W : (W <= 8 ? 8 : 11);
+    constexpr uint32_t from = W == 6 ? 16 : (W == 7 ? 9 : (W == 9 ? 14 : (W == 10 ? 12 : 8)));
+    if (a.m <= stripe_limit<S>() && a.fixed_e >= from) return launch_filter_variant<W, 2, S>(a, stream);
+  }
+  return launch_filter_variant<W, 2>(a, stream);
 }
 
 }  // namespace gk

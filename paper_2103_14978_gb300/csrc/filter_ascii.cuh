@@ -74,7 +74,7 @@ __global__ void __launch_bounds__(kFilterThreads, MinBlocksAscii<W>::value)
     x.rid = a.pair_read[p];
     x.off = a.pair_off[p];
     if (a.pair_e) x.e = a.pair_e[p];
-    x.status = ((uint64_t)x.rid >= a.n_reads || (uint64_t)x.off + a.m > a.ref_len) ? 2 : 0;
+    x.status = (x.rid > a.rid_last || x.off >= a.off_end) ? 2 : 0;
   }
   if (a.err_count) {
     const unsigned bad = __ballot_sync(0xffffffffu, active && x.status == 2);

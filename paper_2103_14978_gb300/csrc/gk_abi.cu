@@ -264,6 +264,7 @@ int gk_filter(gk_ref_t ref, const uint32_t *reads, uint32_t stride_words, uint64
   a.accept = accept_out;
   a.edits = edits_out;
   a.err_count = err_count;
+  a.set_bounds();
   // A genome with N makes a share of windows undefined (about 1 - (1-r)^m
   // for an N density r): filter only the defined pairs, in full warps, when
   // that share (r*m >= 0.05) and the per-pair work repay the queueing.  The
@@ -328,6 +329,7 @@ int gk_filter_sweep(gk_ref_t ref, const uint32_t *reads, uint32_t stride_words, 
   a.accept = accept_out;
   a.edits = edits_out;
   a.err_count = err_count;
+  a.set_bounds();
   // As gk_filter: with a genome dense in N, persistent warps filter only
   // the defined pairs (a sweep is work enough to repay the queueing).
   const bool n_dense = (double)ref->n_undefined * (double)m >= 0.05 * (double)ref->n_bases;
@@ -376,6 +378,7 @@ int gk_filter_ascii(gk_ref_t ref, const uint8_t *ascii, uint64_t ascii_stride, u
   a.accept = accept_out;
   a.edits = edits_out;
   a.err_count = err_count;
+  a.set_bounds();
   g.ascii = ascii;
   g.ascii_stride = ascii_stride;
   g.rows_aligned = (aligned(ascii, 4) && ascii_stride % 4 == 0) ? 1 : 0;

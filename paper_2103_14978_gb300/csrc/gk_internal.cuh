@@ -66,6 +66,15 @@ struct FilterArgs {
   // sweep_hi < fixed_e: one threshold.
   uint32_t sweep_hi;
   uint64_t out_stride;
+  // A pair of a launch with one read length m is valid iff its read id <=
+  // rid_last and its offset < off_end (set_bounds): 32-bit compares.
+  uint32_t rid_last, off_end;
+
+  // From n_reads, ref_len (< 2^32) and m.
+  void set_bounds() {
+    rid_last = n_reads >= (1ull << 32) ? 0xffffffffu : (n_reads ? (uint32_t)(n_reads - 1) : 0u);
+    off_end = n_reads == 0 || ref_len < m ? 0u : (uint32_t)(ref_len - m + 1);
+  }
 };
 
 // Launches the plain filter for words-per-read W = ceil(m/32) (1..16).

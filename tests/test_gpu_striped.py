@@ -40,3 +40,21 @@ def test_sweep_at_stripe_edges(m):
             assert_same((acc[e].cpu().numpy(), dd.edits_u16(ed[e])),
                         oracle_run(w, e, O.RUNS4 if mode == gk.GK_COUNT_RUNS4 else O.POPCOUNT),
                         f"m={m} cands={cands} e={e}")
+
+
+@pytest.mark.parametrize("m", [m for m in EDGES if m >= 65])
+def test_one_threshold_at_stripe_edges(m):
+    """Shift counts around those from which one threshold runs striped, and
+    the largest (30); neighbours that share a read and pairs in random order;
+    the queue of defined pairs."""
+    for cands, n_frac, mode in ((4, 0.0, gk.GK_COUNT_RUNS4), (5, 0.0, gk.GK_COUNT_POPCOUNT),
+                                (6, 0.002, gk.GK_COUNT_RUNS4)):
+        w = small_workload(m, 1501, seed=3500 + m + cands, n_frac=n_frac, read_n_frac=n_frac, cands=cands)
+        if cands == 5:
+            perm = np.random.default_rng(m).permutation(w.n_pairs)
+            w.pair_read, w.pair_off = w.pair_read[perm].copy(), w.pair_off[perm].copy()
+        run = GpuRun(w)
+        for e in (7, 8, 9, 12, 14, 16, 17, 25, 30):
+            assert_same(run.filter(e=e, mode=mode),
+                        oracle_run(w, e, O.RUNS4 if mode == gk.GK_COUNT_RUNS4 else O.POPCOUNT),
+                        f"m={m} cands={cands} e={e}")
