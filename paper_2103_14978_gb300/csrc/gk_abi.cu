@@ -37,10 +37,12 @@ int cuda_check(cudaError_t err, const char *what) {
   return fail(GK_ECUDA, std::string(what) + ": " + cudaGetErrorString(err));
 }
 
-// Variant of the per-pair code for a launch: 2 deferred erosion, 1 exact
-// with every shift below 32, 0 exact for any thresholds.
+// Variant of the per-pair code for a launch: 5 per-pair thresholds (gk_filter
+// with the edge OR), 4 a threshold 0..2 at W <= 4, 3 a sweep, 2 deferred
+// erosion, 1 exact with every shift below 32, 0 exact for any thresholds.
 int filter_variant(const FilterArgs &a, bool pair_k) {
   if (a.out_stride != 0) return 3;  // a threshold sweep (gk_filter_sweep)
+  if (pair_k && a.pair_e && a.edge_on && a.m > 0) return 5;  // sorted by threshold (filter_by_e_kernel)
   // One threshold 0..2 below m, reads of at most 128 bases, no compaction:
   // the two-pairs-per-thread deferred kernel with the shift count fixed at
   // compile time (measured on GB300 at 100 bp against the exact one-pair

@@ -58,3 +58,24 @@ def test_one_threshold_at_stripe_edges(m):
             assert_same(run.filter(e=e, mode=mode),
                         oracle_run(w, e, O.RUNS4 if mode == gk.GK_COUNT_RUNS4 else O.POPCOUNT),
                         f"m={m} cands={cands} e={e}")
+
+
+@pytest.mark.parametrize("m", [1, 2, 31, 33, 96, 100, 126, 127, 150, 156, 157, 254, 255, 300, 349, 512])
+def test_per_pair_thresholds_sorted_in_tiles(m):
+    """Thresholds on both sides of the largest deferred shift count (30) and
+    past m; launches of one pair, a partial warp, whole and partial tiles; N
+    in genome and reads; invalid pairs, counted once."""
+    w = small_workload(m, 5001, seed=3900 + m, n_frac=0.001, read_n_frac=0.001, cands=3, e_rates=(0.02,))
+    rng = np.random.default_rng(m)
+    w.pair_e = rng.choice(np.array([0, 1, 2, 5, 9, 15, 29, 30, 31, 32, 60, 255], np.uint8), w.n_pairs)
+    w.pair_read[rng.integers(0, w.n_pairs, 9)] = w.n_reads
+    run = GpuRun(w)
+    want = oracle_run(w)
+    r, p = run.reads, run.pairs
+    for n in (1, 31, 128, 129, 1000, 5001):
+        err = torch.zeros(1, dtype=torch.int32, device="cuda")
+        acc, ed = gk.gk_filter(run.ref, r.packed, r.stride_words, r.n_reads, r.nflag, m, p.pair_read[:n],
+                               p.pair_off[:n], p.pair_e[:n], err_count=err)
+        torch.cuda.synchronize()
+        assert_same((acc.cpu().numpy(), dd.edits_u16(ed)), (want[0][:n], want[1][:n]), f"m={m} n={n}")
+        assert int(err.item()) == int((want[1][:n] == O.INVALID).sum())
