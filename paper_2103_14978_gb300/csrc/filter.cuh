@@ -1140,7 +1140,10 @@ __global__ void __launch_bounds__(kFilterThreads, S == 5 ? 6 : MinBlocks2<W>::va
   const int s1 = act1 ? pair_status<W>(a, x1) : -1;
   if (s0 > 0) write_trivial(a, p0, s0);
   if (s1 > 0) write_trivial(a, p1, s1);
-  if (s0 == 0 && s1 == 0 && x0.rid == x1.rid) {
+  // One form per warp, as in sweep_pair2_kernel.
+  const bool shared = s0 == 0 && s1 == 0 && x0.rid == x1.rid;
+  if (!__any_sync(0xffffffffu, !shared && (s0 == 0 || s1 == 0))) {
+    if (!shared) return;
     const uint32_t K = KC >= 0 ? (uint32_t)KC : min(a.fixed_e, a.m - 1);
     uint32_t count[2];
     if constexpr (S > 0) {
@@ -1207,7 +1210,12 @@ __global__ void __launch_bounds__(kFilterThreads, S == 5 ? 6 : 8) sweep_pair2_ke
   const int s1 = act1 ? pair_status<W>(a, x1) : -1;
   if (s0 > 0) write_trivial<true>(a, p0, s0);
   if (s1 > 0) write_trivial<true>(a, p1, s1);
-  if (s0 == 0 && s1 == 0 && x0.rid == x1.rid) {
+  // One form per warp: pairs of different reads in a few lanes (a read's
+  // candidates ending on an odd pair) would make it run both (10M pairs of 100
+  // bp, 13 candidates per read, e = 0..10: 0.85 -> 0.48 ms).
+  const bool shared = s0 == 0 && s1 == 0 && x0.rid == x1.rid;
+  if (!__any_sync(0xffffffffu, !shared && (s0 == 0 || s1 == 0))) {
+    if (!shared) return;
     const uint32_t e_lo = a.fixed_e, e_hi = a.sweep_hi, kmax = a.m - 1;
     const uint32_t Klo = min(e_lo, kmax), Khi = min(e_hi, kmax);
     // Pairs 2t and 2t+1 are adjacent in every row: packed stores when the
@@ -1487,24 +1495,38 @@ cudaError_t launch_filter_variant(const FilterArgs &a, cudaStream_t stream) {
 }
 
 // Launches the threshold sweep over reads of W = ceil(m/32) words: striped
-// where the stripes hold the read (stripe_limit) and beat the linear form.
-// Measured on GB300, launches alone, linear -> striped: 76 bp (S = 3) at e =
-// 0..8 0.230 -> 0.166 ms; 200 bp (S = 8) at 0..20 0.599 -> 0.443; 300 bp (S =
-// 11) at 0..30 1.146 -> 0.958; 100, 150 and 250 bp beside striped_exact.  W =
-// 1 needs one linear word and three stripes; from W = 11 on the stripes spill.
+// where the stripes hold the read (stripe_limit) and beat the linear form at
+// the sweep's largest shift count, also where neighbouring pairs name
+// different reads.  Measured on GB300, launches alone from e = 0, linear /
+// striped in us, pairs in fours of one read (in brackets: each its own read):
+//   50 bp  8M  e 1  90 / 88 (122 / 119), 5 190 / 168 (224 / 205)
+//   76 bp  8M  e 1 105 / 96 (142 / 135), 8 344 / 246 (424 / 301)
+//   96 bp  8M  e 2 138 / 136 (172 / 178), 3 172 / 158, 10 416 / 305
+//   100 bp 10M e 1 160 / 158 (240 / 224), 5 345 / 248 (439 / 316), 10 603 / 383
+//   128 bp 8M  e 2 161 / 166 (222 / 221), 6 322 / 298 (409 / 346)
+//   150 bp 6M  e 1 121 / 109 (125 / 154), 3 191 / 148 (193 / 195), 15 686 / 438
+//   160 bp 6M  e 3 191 / 252, 8 396 / 397, 16 730 / 645
+//   170 bp 5M  e 3 177 / 221, 9 407 / 379, 17 719 / 605
+//   200 bp 4M  e 2 135 / 158, 4 201 / 193, 20 773 / 519
+//   250 bp 4M  e 2 158 / 162, 5 263 / 222, 25 1062 / 660
+//   280 bp 3M  e 6 248 / 267, 14 514 / 496
+//   300 bp 3M  e 6 269 / 279, 15 594 / 533, 30 1136 / 891
+// W = 1 needs one linear word and three stripes; from W = 11 the stripes spill.
 template <int W>
 cudaError_t launch_sweep(const FilterArgs &a, cudaStream_t stream) {
-  if constexpr (W == 1 || W > 10) {
-    return launch_filter_variant<W, 3>(a, stream);
-  } else {
+  if constexpr (W >= 2 && W <= 10) {
     constexpr int S0 = W <= 3 ? 3 : (W <= 5 ? W : (W <= 8 ? 8 : 11));
-    constexpr int S1 = W == 3 ? 4 : (W == 4 ? 5 : (W == 5 ? 8 : 0));  // 0: linear
-    if (a.m <= stripe_limit<S0>()) return launch_filter_variant<W, 3, S0>(a, stream);
-    if constexpr (32 * W <= stripe_limit<S0>())
-      return cudaErrorInvalidValue;
-    else
-      return launch_filter_variant<W, 3, S1>(a, stream);
+    constexpr int S1 = W == 3 ? 4 : (W == 4 ? 5 : (W == 5 ? 8 : 0));  // reads S0 does not hold
+    constexpr uint32_t from0 = W <= 4 ? 0 : W == 5 ? 3 : W == 6 ? 9 : W == 7 ? 4 : W == 8 ? 3 : W == 9 ? 14 : 9;
+    constexpr uint32_t from1 = W == 5 ? 10 : 3;
+    const uint32_t K = min(a.sweep_hi, a.m - 1);
+    if (a.m <= stripe_limit<S0>()) {
+      if (K >= from0) return launch_filter_variant<W, 3, S0>(a, stream);
+    } else if constexpr (S1 > 0) {
+      if (K >= from1) return launch_filter_variant<W, 3, S1>(a, stream);
+    }
   }
+  return launch_filter_variant<W, 3>(a, stream);
 }
 
 // Launches VARIANT 2 (one threshold, shift count 2 .. 30, edge OR on) over
