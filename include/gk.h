@@ -303,8 +303,8 @@ int gk_filter_sliced_sweep(const void *sliced, uint64_t sliced_cap, uint64_t n_p
 /* Tiling of the batched filter (chosen by the autotuner). */
 typedef struct {
   uint32_t words_per_thread; /* words of a pair held per lane: 2, 3, 4, 6 or 8;
-                                1 = a whole pair per lane for reads up to 256
-                                bases (4 words per lane above) */
+                                1 = a whole pair per lane (the other fields are
+                                then checked and not used) */
   uint32_t tile_pairs;       /* pairs per tile (work unit of a warp), 32..65536 */
   uint32_t blocks_per_sm;    /* persistent grid = SM count x this, 1..32 */
   uint32_t warps_per_block;  /* 1..8 */
@@ -333,9 +333,11 @@ uint64_t gk_filter_batched_workspace(uint64_t n_pairs);
  *               n_pairs) bytes, 256-byte aligned, owned by the caller; its
  *               contents need no initialisation and are garbage afterwards;
  *               two calls in flight at once need two workspaces
- * Enqueues a memset, three planning kernels (classify, scan, scatter) and the
- * persistent filter kernel on `stream`; everything is stream-ordered and can
- * be captured in a CUDA graph.  n_pairs must be < 2^32.
+ * With words_per_thread 1 enqueues one kernel up to 2 million pairs, above that
+ * a planning kernel and one filter kernel per range of read lengths; else a
+ * memset, three planning kernels (classify, scan, scatter) and the persistent
+ * filter kernel.  Everything is stream-ordered and can be captured in a CUDA
+ * graph.  n_pairs must be < 2^32.
  */
 int gk_filter_batched(gk_ref_t ref, const uint32_t *reads, uint32_t stride_words,
                       uint64_t n_reads, const uint16_t *read_len,

@@ -136,8 +136,6 @@ __global__ void __launch_bounds__(1024) scan_kernel(const BatchArgs a) {
     a.s.tile_base[kKeys] = bt;
     a.s.counters[0] = 0;
     a.s.counters[1] = bt;
-    a.s.counters[2] = 0;
-    a.s.counters[3] = 0;
   }
 }
 
@@ -208,9 +206,10 @@ BatchScratch batch_scratch_layout(void *base, uint64_t n_pairs) {
   return s;
 }
 
-cudaError_t launch_whole_w1_8(const BatchArgs &a, uint32_t sms, uint32_t bpsm, uint32_t wpb, cudaStream_t s);
-cudaError_t launch_whole_w9_12(const BatchArgs &a, uint32_t sms, uint32_t bpsm, uint32_t wpb, cudaStream_t s);
-cudaError_t launch_whole_w13_16(const BatchArgs &a, uint32_t sms, uint32_t bpsm, uint32_t wpb, cudaStream_t s);
+cudaError_t launch_tiles_w4(const BatchArgs &a, cudaStream_t s);
+cudaError_t launch_tiles_w8(const BatchArgs &a, cudaStream_t s);
+cudaError_t launch_tiles_w10(const BatchArgs &a, cudaStream_t s);
+cudaError_t launch_tiles_w16(const BatchArgs &a, cudaStream_t s);
 cudaError_t launch_persistent_wpt2(const BatchArgs &a, uint32_t grid, uint32_t wpb, cudaStream_t s);
 cudaError_t launch_persistent_wpt3(const BatchArgs &a, uint32_t grid, uint32_t wpb, cudaStream_t s);
 cudaError_t launch_persistent_wpt4(const BatchArgs &a, uint32_t grid, uint32_t wpb, cudaStream_t s);
@@ -220,6 +219,11 @@ cudaError_t launch_persistent_wpt8(const BatchArgs &a, uint32_t grid, uint32_t w
 cudaError_t launch_batched(int wpt, const BatchArgs &a, uint32_t blocks_per_sm, uint32_t warps_per_block,
                            cudaStream_t stream) {
   if (a.f.n_pairs == 0) return cudaSuccess;
+  if (wpt == 1) {  // one pair per lane: sorted in tiles, one launch
+    const uint32_t sw = a.f.stride_words;
+    return sw <= 4 ? launch_tiles_w4(a, stream) : sw <= 8 ? launch_tiles_w8(a, stream)
+           : sw <= 10 ? launch_tiles_w10(a, stream) : launch_tiles_w16(a, stream);
+  }
   cudaError_t err = cudaMemsetAsync(a.s.hist, 0, sizeof(uint32_t) * kKeys, stream);
   if (err != cudaSuccess) return err;
   const unsigned cblocks = (unsigned)((a.f.n_pairs + kClassifyChunk - 1) / kClassifyChunk);
@@ -233,15 +237,6 @@ cudaError_t launch_batched(int wpt, const BatchArgs &a, uint32_t blocks_per_sm, 
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   const uint32_t grid = (uint32_t)sms * blocks_per_sm;
-  if (wpt == 1) {
-    // One pair per lane: three W ranges, widest first; each launch drains its
-    // own range of tiles.
-    const uint32_t n = (uint32_t)sms;
-    err = launch_whole_w13_16(a, n, blocks_per_sm, warps_per_block, stream);
-    if (err == cudaSuccess) err = launch_whole_w9_12(a, n, blocks_per_sm, warps_per_block, stream);
-    if (err == cudaSuccess) err = launch_whole_w1_8(a, n, blocks_per_sm, warps_per_block, stream);
-    return err;
-  }
   switch (wpt) {
     case 2: return launch_persistent_wpt2(a, grid, warps_per_block, stream);
     case 3: return launch_persistent_wpt3(a, grid, warps_per_block, stream);
