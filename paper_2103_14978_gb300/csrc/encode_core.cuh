@@ -5,6 +5,8 @@
 
 #include <cstdint>
 
+#include "stripe.cuh"
+
 namespace gk {
 
 // Four ASCII bytes -> 4 bits each of the high plane, the low plane and the
@@ -47,32 +49,40 @@ __device__ __forceinline__ void encode32(const uint32_t (&wb)[8], uint32_t nvali
 // A full word (32 bytes) -> its planes and whether any byte is not A/C/G/T
 // (either case).  Per pair of 4-byte words, bit 2
 // (high plane) and bit 1 XOR bit 2 (low plane) of each byte are gathered by
-// one multiply each into the top byte of a product, the first word's 4 bits
-// at bits 24..27 and the second's at 28..31 (the magic shifted by 4; no
-// other partial product lands in that byte, so the two products are ORed);
+// one multiply-add each into the top byte of a sum, the first word's 4 bits
+// at bits 24..27 and the second's at 28..31 (the magic shifted by 4; all 20
+// partial products are distinct bits, so the sum carries nothing);
 // three byte permutes assemble the four top bytes into the plane word.
-// Validity looks up the letter a byte's bits 2 and 1 name ("A", "C", "T",
-// "G" for 00, 01, 10, 11) with two byte permutes and compares it with the
-// case-folded byte.  bad != 0: re-encode with encode32 (codes 00 for the
-// undefined bytes).
+//
+// Validity is a relation between a byte's bits b7..b0 that holds for just the
+// eight letters: b7 = 0, b6 = 1, b3 = 0, b4 = b2 & ~b1, b0 = ~b4 (b5 is the
+// case).  Left shifts bring b2, b1 and b0 to b4's place (in their own byte);
+// the outcomes of all bytes are ORed and tested once.  Shifts and products run
+// on the multiply-add pipe beside 5.5 logic ops per 4 bytes on the ALU pipe
+// (looking up the letter a byte's bits name, two byte permutes and six logic
+// ops, took 16): 5M reads of 100 bases 0.160 -> 0.132 ms.
+// bad != 0: re-encode with encode32 (codes 00 for the undefined bytes).
 __device__ __forceinline__ void encode32_full(const uint32_t (&wb)[8], uint32_t &hi, uint32_t &lo, uint32_t &bad) {
   constexpr uint32_t kM = 0x00408102u;  // bit 2 of byte k -> bit 24 + k
   uint32_t yh[4], yl[4];
-  bad = 0;
+  uint32_t any = 0u, all = 0xffffffffu, wrong = 0u;
 #pragma unroll
   for (int p = 0; p < 4; ++p) {
     const uint32_t c0 = wb[2 * p], c1 = wb[2 * p + 1];
-    yh[p] = ((c0 & 0x04040404u) * kM) | ((c1 & 0x04040404u) * (kM << 4));
-    yl[p] = (((c0 ^ (c0 << 1)) & 0x04040404u) * kM) | (((c1 ^ (c1 << 1)) & 0x04040404u) * (kM << 4));
+    yh[p] = (c1 & 0x04040404u) * (kM << 4) + (c0 & 0x04040404u) * kM;
+    yl[p] = ((c1 ^ (c1 << 1)) & 0x04040404u) * (kM << 4) + ((c0 ^ (c0 << 1)) & 0x04040404u) * kM;
+    uint32_t w[2];
 #pragma unroll
     for (int q = 0; q < 2; ++q) {
       const uint32_t c = wb[2 * p + q];
-      const uint32_t idx = (c >> 1) & 0x03030303u;
-      const uint32_t sel = __byte_perm(idx | (idx >> 4), 0u, 0x4420u);
-      const uint32_t expect = __byte_perm(0x47544341u, 0u, sel);  // 'A' 'C' 'T' 'G'
-      bad |= (c ^ expect) & 0xDFDFDFDFu;
+      const uint32_t u = lop3<0xB4>(c, c << 2, c << 3);  // b4 ^ (b2 & ~b1): a ^ (b & ~c)
+      w[q] = lop3<0xF9>(u, c, c << 4);                   // u | ~(b4 ^ b0)
     }
+    wrong = lop3<0xFE>(wrong, w[0], w[1]);
+    any = lop3<0xFE>(any, c0, c1);
+    all = lop3<0x80>(all, c0, c1);
   }
+  bad = (wrong & 0x10101010u) | (any & 0x88888888u) | (~all & 0x40404040u);
   hi = __byte_perm(__byte_perm(yh[0], yh[1], 0x0073u), __byte_perm(yh[2], yh[3], 0x0073u), 0x5410u);
   lo = __byte_perm(__byte_perm(yl[0], yl[1], 0x0073u), __byte_perm(yl[2], yl[3], 0x0073u), 0x5410u);
 }
