@@ -232,12 +232,12 @@ cudaError_t launch_sliced_filter(int K, const SlicedArgs &a, cudaStream_t stream
 }
 
 cudaError_t launch_sliced_sweep(int klo, int khi, const SlicedArgs &a, cudaStream_t stream) {
-  if (!sliced_sweep_range(klo, khi)) return cudaErrorInvalidValue;
+  if (klo != (khi <= 5 ? 0 : 6)) return cudaErrorInvalidValue;
   switch (a.m) {
-    case 100: return launch_sliced_sweep_m100(klo, a, stream);
-    case 150: return launch_sliced_sweep_m150(klo, a, stream);
-    case 250: return launch_sliced_sweep_m250(klo, a, stream);
-    default: return launch_sliced_sweep_m0(klo, a, stream);
+    case 100: return launch_sliced_sweep_m100(khi, a, stream);
+    case 150: return launch_sliced_sweep_m150(khi, a, stream);
+    case 250: return launch_sliced_sweep_m250(khi, a, stream);
+    default: return launch_sliced_sweep_m0(khi, a, stream);
   }
 }
 
@@ -379,7 +379,7 @@ int gk_filter_sliced_sweep(const void *sliced, uint64_t sliced_cap, uint64_t n_p
     const uint32_t K = e < m - 1 ? e : m - 1;
     int klo = -1, khi = -1;
     uint32_t last = e;
-    if (e <= m - 1 && gk::sliced_sweep_cover((int)K, &klo, &khi)) {
+    if (e <= m - 1 && gk::sliced_sweep_cover((int)K, (int)k_hi, &klo, &khi)) {
       last = (uint32_t)khi;
       if (last > e_hi) last = e_hi;
       if (last > m - 1) last = m - 1;

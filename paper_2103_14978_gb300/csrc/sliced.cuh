@@ -638,36 +638,32 @@ __host__ __device__ __forceinline__ void sliced_sweep_group(const SlicedArgs &a,
 }
 
 // Compiled ranges of shift counts of the sweep kernels (sliced_sweep_m*.cu).
-__host__ __device__ __forceinline__ bool sliced_sweep_range(int klo, int khi) {
-  return (klo == 0 && khi == 5) || (klo == 6 && khi == 10);
-}
-// The compiled range holding shift count K, if any.
-__host__ __device__ __forceinline__ bool sliced_sweep_cover(int K, int *klo, int *khi) {
-  if (K >= 0 && K <= 5) {
-    *klo = 0;
-    *khi = 5;
-    return true;
-  }
-  if (K >= 6 && K <= 10) {
-    *klo = 6;
-    *khi = 10;
-    return true;
-  }
-  return false;
+// A range costs all its shift counts, written or not: 4 (2 KHI + 1) logic ops
+// per position for the masks and about 13 per shift count for erosion and
+// count, so a sweep that ends at 7 or 8 has a range of its own (5M pairs of 150
+// bp, e = 0..7: 430 us with 6 and 7 out of the range 6..10, 341 out of 6..7).
+//
+// The range for shift counts K .. last of a sweep, or its first part: 0..5, or
+// 6 to the smallest compiled end at or above last.
+__host__ __device__ __forceinline__ bool sliced_sweep_cover(int K, int last, int *klo, int *khi) {
+  if (K < 0 || K > 10) return false;
+  *klo = K <= 5 ? 0 : 6;
+  *khi = K <= 5 ? 5 : (last <= 7 ? 7 : (last == 8 ? 8 : 10));
+  return true;
 }
 
 // Launchers (sliced.cu, sliced_m*_k*.cu, sliced_sweep_m*.cu).
 cudaError_t launch_slice(const SliceArgs &a, uint32_t *err_count, cudaStream_t stream);
 // One threshold: shift count K = min(e, m-1).
 cudaError_t launch_sliced_filter(int K, const SlicedArgs &a, cudaStream_t stream);
-// A compiled range of shift counts [klo, khi] (sliced_sweep_ranges) with
+// A compiled range of shift counts [klo, khi] (sliced_sweep_cover) with
 // results for a.k_first .. a.k_last inside it.
 cudaError_t launch_sliced_sweep(int klo, int khi, const SlicedArgs &a, cudaStream_t stream);
 #define GK_SLICED_LAUNCHERS(M)                                                                  \
   cudaError_t launch_sliced_m##M##_k0_5(int K, const SlicedArgs &a, cudaStream_t stream);  \
   cudaError_t launch_sliced_m##M##_k6_10(int K, const SlicedArgs &a, cudaStream_t stream); \
   cudaError_t launch_sliced_m##M##_k11_15(int K, const SlicedArgs &a, cudaStream_t stream); \
-  cudaError_t launch_sliced_sweep_m##M(int klo, const SlicedArgs &a, cudaStream_t stream);
+  cudaError_t launch_sliced_sweep_m##M(int khi, const SlicedArgs &a, cudaStream_t stream);
 GK_SLICED_LAUNCHERS(0)
 GK_SLICED_LAUNCHERS(100)
 GK_SLICED_LAUNCHERS(150)

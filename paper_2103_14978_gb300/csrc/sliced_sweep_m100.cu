@@ -4,10 +4,12 @@
 
 namespace gk {
 
-cudaError_t launch_sliced_sweep_m100(int klo, const SlicedArgs &a, cudaStream_t stream) {
-  switch (klo) {
-    case 0: return launch_sliced_range<0, 5, 100>(a, stream);
-    case 6: return launch_sliced_range<6, 10, 100>(a, stream);
+cudaError_t launch_sliced_sweep_m100(int khi, const SlicedArgs &a, cudaStream_t stream) {
+  switch (khi) {
+    case 5: return launch_sliced_range<0, 5, 100>(a, stream);
+    case 7: return launch_sliced_range<6, 7, 100>(a, stream);
+    case 8: return launch_sliced_range<6, 8, 100>(a, stream);
+    case 10: return launch_sliced_range<6, 10, 100>(a, stream);
     default: return cudaErrorInvalidValue;
   }
 }

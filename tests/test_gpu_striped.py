@@ -79,3 +79,18 @@ def test_per_pair_thresholds_sorted_in_tiles(m):
         torch.cuda.synchronize()
         assert_same((acc.cpu().numpy(), dd.edits_u16(ed)), (want[0][:n], want[1][:n]), f"m={m} n={n}")
         assert int(err.item()) == int((want[1][:n] == O.INVALID).sum())
+
+
+@pytest.mark.parametrize("m", [8, 9, 100, 120, 150, 250])
+@pytest.mark.parametrize("e_lo,e_hi", [(0, 7), (5, 8), (6, 7), (7, 8), (6, 9)])
+def test_sliced_sweep_range_ends(m, e_lo, e_hi):
+    """Sliced sweeps that end at 7, 8 and above; thresholds past m - 1."""
+    w = small_workload(m, 700, seed=3300 + m)
+    run = GpuRun(w)
+    r = run.reads
+    buf = gk.gk_slice(run.ref, r.packed, r.stride_words, r.n_reads, r.nflag, m, run.pairs.pair_read,
+                      run.pairs.pair_off)
+    acc, ed = gk.gk_filter_sliced_sweep(buf, w.n_pairs, m, e_lo, e_hi)
+    torch.cuda.synchronize()
+    for e in range(e_lo, e_hi + 1):
+        assert_same((acc[e - e_lo].cpu().numpy(), dd.edits_u16(ed[e - e_lo])), oracle_run(w, e), f"m={m} e={e}")
