@@ -33,6 +33,7 @@
 #include <atomic>
 
 #include "gk_internal.cuh"
+#include "overlap.cuh"
 #include "stripe.cuh"
 
 namespace gk {
@@ -861,9 +862,14 @@ __device__ __forceinline__ void filter_and_write(const FilterArgs &a, uint64_t p
     sweep_and_write<W, S>(a, p, x);
   } else {
     uint32_t count;
-    if constexpr (S > 0)
+    if constexpr (S > 0) {
       count = filter_loaded_striped<W, S>(a, x, min(a.fixed_e, a.m - 1));
-    else
+    } else if constexpr (S < 0) {
+      uint32_t rh[W], rl[W], gh[1][W], gl[1][W], c[1];
+      pair_planes<W>(x, rh, rl, gh[0], gl[0]);
+      overlap_counts<W, 1, -1>(a.m, min(a.fixed_e, a.m - 1), a.count_mode, rh, rl, gh, gl, c);
+      count = c[0];
+    } else
       count = VARIANT == 4   ? filter_loaded_deferred<W, true>(a, x)
               : VARIANT == 2 ? filter_loaded_deferred<W>(a, x)
                              : filter_loaded<W, VARIANT == 1>(a, x);
@@ -944,7 +950,8 @@ constexpr size_t compact_smem_bytes() {
 // VARIANT 0: any thresholds; 1: every shift count of the launch is < 32;
 // 2: edge OR on and one threshold in 2..30, deferred erosion; 3: edge OR on,
 // a sweep of thresholds up to 30 (sweep_and_write).  2 and 3 are striped in S
-// words or, S = 0, linear.
+// words (S > 0), 2 and 4 in overlapping words (S = -1, shift counts up to
+// kOverlapMax) or linear (S = 0).
 //
 // COMPACT false: one thread per pair.  COMPACT true (inputs with many
 // undefined pairs): persistent warps take 32 pairs at a time (their ids
@@ -1115,7 +1122,7 @@ struct MinBlocks2 {
 // the end corrections of K = 0 vanish.
 //
 // S > 0: striped; of pairs that do not share a read the second is then loaded
-// anew, as in the sweep.
+// anew, as in the sweep.  S = -1: in overlapping words (overlap.cuh).
 template <int W, int VARIANT, int KC = -1, int S = 0>
 __global__ void __launch_bounds__(kFilterThreads, S == 5 ? 6 : MinBlocks2<W>::value)
     filter_pair2_kernel(const FilterArgs a) {
@@ -1155,7 +1162,10 @@ __global__ void __launch_bounds__(kFilterThreads, S == 5 ? 6 : MinBlocks2<W>::va
       uint32_t rh[W], rl[W], gh[2][W], gl[2][W];
       pair_planes<W>(x0, rh, rl, gh[0], gl[0]);
       window_planes<W>(x1, gh[1], gl[1]);
-      deferred_counts<W, 2, (KC >= 0)>(a, a.m, K, rh, rl, gh, gl, count);
+      if constexpr (S < 0)
+        overlap_counts<W, 2, KC>(a.m, K, a.count_mode, rh, rl, gh, gl, count);
+      else
+        deferred_counts<W, 2, (KC >= 0)>(a, a.m, K, rh, rl, gh, gl, count);
     }
     // The two pairs are adjacent: one 2-byte accept store and one 4-byte
     // count store when the buffers allow it.
@@ -1176,8 +1186,8 @@ __global__ void __launch_bounds__(kFilterThreads, S == 5 ? 6 : MinBlocks2<W>::va
       filter_and_write<W, VARIANT, S>(a, p0 + j, x0);
     }
   } else {
-    if (s0 == 0) filter_and_write<W, VARIANT>(a, p0, x0);
-    if (s1 == 0) filter_and_write<W, VARIANT>(a, p1, x1);
+    if (s0 == 0) filter_and_write<W, VARIANT, S>(a, p0, x0);
+    if (s1 == 0) filter_and_write<W, VARIANT, S>(a, p1, x1);
   }
 }
 
@@ -1439,9 +1449,9 @@ cudaError_t launch_filter_variant(const FilterArgs &a, cudaStream_t stream) {
         if constexpr (VARIANT == 4) {
           // shift count = the threshold, 0..2, below m (checked by the caller)
           switch (a.fixed_e) {
-            case 0: filter_pair2_kernel<W, 4, 0><<<grid, kFilterThreads, 0, stream>>>(a); break;
-            case 1: filter_pair2_kernel<W, 4, 1><<<grid, kFilterThreads, 0, stream>>>(a); break;
-            case 2: filter_pair2_kernel<W, 4, 2><<<grid, kFilterThreads, 0, stream>>>(a); break;
+            case 0: filter_pair2_kernel<W, 4, 0, S><<<grid, kFilterThreads, 0, stream>>>(a); break;
+            case 1: filter_pair2_kernel<W, 4, 1, S><<<grid, kFilterThreads, 0, stream>>>(a); break;
+            case 2: filter_pair2_kernel<W, 4, 2, S><<<grid, kFilterThreads, 0, stream>>>(a); break;
             default: return cudaErrorInvalidValue;
           }
         } else {
@@ -1542,14 +1552,39 @@ cudaError_t launch_sweep(const FilterArgs &a, cudaStream_t stream) {
 // 250 bp K = 5 188 / 209, 8 257 / 242, 25 687 / 473; 3M of 280 bp K = 14 345 /
 // 326; of 300 bp K = 9 258 / 258, 15 400 / 347; 128 and 160 bp (S = 5 and 8 with
 // 20 rows) no faster up to K = 16.
+//
+// Up to shift count 7 in overlapping words where they hold the read (m <= 30 W)
+// and W <= 8, ordinary / overlapping words in us on the same launches: 50 bp K =
+// 2 97 / 91, 7 150 / 134; 76 bp K = 2 112 / 107, 7 193 / 168; 100 bp K = 3 187 /
+// 174, 5 234 / 209, 7 290 / 253; 150 bp K = 2 135 / 135, 5 197 / 184; 200 bp K =
+// 2 123 / 111, 7 209 / 187; 240 bp K = 3 156 / 138, 7 232 / 205.
+template <int W>
+__host__ constexpr uint32_t single_striped_from() {
+  return W == 6 ? 16 : (W == 7 ? 9 : (W == 9 ? 14 : (W == 10 ? 12 : 8)));
+}
+template <int W>
+__host__ bool single_overlaps(const FilterArgs &a) {
+  return W >= 2 && W <= 8 && a.m <= overlap_limit<W>() && a.fixed_e <= kOverlapMax && (W != 5 || a.fixed_e >= 3);
+}
 template <int W>
 cudaError_t launch_single(const FilterArgs &a, cudaStream_t stream) {
+  if constexpr (W >= 2 && W <= 8)
+    if (single_overlaps<W>(a)) return launch_filter_variant<W, 2, -1>(a, stream);
   if constexpr (W >= 3 && W <= 10) {
     constexpr int S = W <= 5 ? W : (W <= 8 ? 8 : 11);
-    constexpr uint32_t from = W == 6 ? 16 : (W == 7 ? 9 : (W == 9 ? 14 : (W == 10 ? 12 : 8)));
-    if (a.m <= stripe_limit<S>() && a.fixed_e >= from) return launch_filter_variant<W, 2, S>(a, stream);
+    if (a.m <= stripe_limit<S>() && a.fixed_e >= single_striped_from<W>())
+      return launch_filter_variant<W, 2, S>(a, stream);
   }
   return launch_filter_variant<W, 2>(a, stream);
+}
+
+// VARIANT 4 (thresholds 0 .. 2, W <= 4): 100 bp K = 0 113 / 112, 1 135 / 130, 2 158
+// / 148 us for 10M pairs.
+template <int W>
+cudaError_t launch_small(const FilterArgs &a, cudaStream_t stream) {
+  if constexpr (W >= 2 && W <= 4)
+    if (a.m <= overlap_limit<W>()) return launch_filter_variant<W, 4, -1>(a, stream);
+  return launch_filter_variant<W, 4>(a, stream);
 }
 
 // Launches per-pair thresholds (edge OR on, m > 0).  Tiles shrink with the

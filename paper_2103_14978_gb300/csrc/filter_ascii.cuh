@@ -91,7 +91,7 @@ struct MinBlocksAscii {
   static constexpr int value = W <= 2 ? 10 : (W <= 4 ? 8 : MinBlocks<W, false>::value);
 };
 
-template <int W, int VARIANT>
+template <int W, int VARIANT, int S = 0>
 __global__ void __launch_bounds__(kFilterThreads, MinBlocksAscii<W>::value)
     filter_ascii_kernel(const AsciiArgs g) {
   const FilterArgs &a = g.f;
@@ -172,13 +172,20 @@ __global__ void __launch_bounds__(kFilterThreads, MinBlocksAscii<W>::value)
     write_trivial(a, p, status);
     return;
   }
-  filter_and_write<W, VARIANT>(a, p, x);
+  filter_and_write<W, VARIANT, S>(a, p, x);
 }
 
-template <int W, int VARIANT>
+template <int W, int VARIANT, int S = 0>
 cudaError_t launch_filter_ascii_variant(const AsciiArgs &g, cudaStream_t stream) {
+  // One threshold, deferred erosion: the same forms as gk_filter's (launch_single).
+  if constexpr (VARIANT == 2 && S == 0) {
+    if constexpr (W >= 2 && W <= 8)
+      if (single_overlaps<W>(g.f)) return launch_filter_ascii_variant<W, 2, -1>(g, stream);
+    if constexpr (W == 4 || W == 5 || W == 8)
+      if (g.f.m <= stripe_limit<W>() && g.f.fixed_e >= 10) return launch_filter_ascii_variant<W, 2, W>(g, stream);
+  }
   const unsigned blocks = (unsigned)((g.f.n_pairs + kFilterThreads - 1) / kFilterThreads);
-  filter_ascii_kernel<W, VARIANT><<<blocks, kFilterThreads, 0, stream>>>(g);
+  filter_ascii_kernel<W, VARIANT, S><<<blocks, kFilterThreads, 0, stream>>>(g);
   return cudaGetLastError();
 }
 

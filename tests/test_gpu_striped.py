@@ -94,3 +94,25 @@ def test_sliced_sweep_range_ends(m, e_lo, e_hi):
     torch.cuda.synchronize()
     for e in range(e_lo, e_hi + 1):
         assert_same((acc[e - e_lo].cpu().numpy(), dd.edits_u16(ed[e - e_lo])), oracle_run(w, e), f"m={m} e={e}")
+
+
+@pytest.mark.parametrize("m", [33, 59, 60, 61, 65, 89, 90, 91, 97, 101, 119, 120, 121, 129, 149, 150, 151, 161, 180, 181,
+                               193, 210, 225, 240, 241])
+def test_overlapping_words_at_their_limits(m):
+    """Every shift count of the overlapping words and the first beyond, at
+    read lengths around those W words hold; neighbours that share a read and
+    pairs in random order; packed reads and ASCII rows."""
+    for cands, mode in ((4, gk.GK_COUNT_RUNS4), (5, gk.GK_COUNT_POPCOUNT)):
+        w = small_workload(m, 1203, seed=3700 + m + cands, cands=cands)
+        if cands == 5:
+            perm = np.random.default_rng(m).permutation(w.n_pairs)
+            w.pair_read, w.pair_off = w.pair_read[perm].copy(), w.pair_off[perm].copy()
+        run = GpuRun(w)
+        asc = torch.from_numpy(np.ascontiguousarray(w.reads)).cuda()
+        for e in (0, 1, 2, 3, 5, 7, 8, 10):
+            want = oracle_run(w, e, O.RUNS4 if mode == gk.GK_COUNT_RUNS4 else O.POPCOUNT)
+            assert_same(run.filter(e=e, mode=mode), want, f"m={m} cands={cands} e={e}")
+            acc, ed = gk.gk_filter_ascii(run.ref, asc, w.stride, w.n_reads, m, run.pairs.pair_read, run.pairs.pair_off,
+                                         e, count_mode=mode)
+            torch.cuda.synchronize()
+            assert_same((acc.cpu().numpy(), dd.edits_u16(ed)), want, f"ascii m={m} cands={cands} e={e}")
