@@ -117,6 +117,8 @@ class GKError(RuntimeError):
 def lib() -> ctypes.CDLL:
     """The loaded libgk.so.  Raises if it has not been built."""
     global _lib
+    if _lib is not None:  # set once, after every signature
+        return _lib
     with _lock:
         if _lib is None:
             if not os.path.exists(LIB_PATH):
@@ -141,9 +143,16 @@ def _check(rc: int):
         raise GKError(rc, lib().gk_last_error().decode())
 
 
+# The current stream's handle, without the stream object that
+# torch.cuda.current_stream() builds around it (2.9 us a call, this 0.3 us).
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+
+
 def _stream(stream) -> int:
     if stream is None:
-        return torch.cuda.current_stream().cuda_stream
+        if _raw_stream is None or not torch.cuda.is_initialized():
+            return torch.cuda.current_stream().cuda_stream
+        return _raw_stream(torch._C._cuda_getDevice())
     if isinstance(stream, torch.cuda.Stream):
         return stream.cuda_stream
     return int(stream)
@@ -154,7 +163,7 @@ def _dptr(t: torch.Tensor | None, dtype: torch.dtype, name: str, numel: int | No
         return None
     if not isinstance(t, torch.Tensor) or not t.is_cuda:
         raise TypeError(f"{name} must be a CUDA tensor")
-    if t.dtype != dtype or not t.is_contiguous():
+    if t.dtype is not dtype or not t.is_contiguous():
         raise TypeError(f"{name} must be a contiguous {dtype} tensor")
     if numel is not None and t.numel() < numel:
         raise ValueError(f"{name} holds {t.numel()} elements, needs {numel}")
