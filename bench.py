@@ -107,8 +107,9 @@ def sliced_bytes_per_pair(m: int) -> float:
 
 
 # Shift-count ranges the library's sweep kernels filter in one launch each
-# (gk_filter_sliced_sweep); a threshold outside them is a single launch.
-SWEEP_RANGES = ((0, 5), (6, 10))
+# (gk_filter_sliced_sweep); of those that hold a sweep's part the first whose
+# end reaches it; a threshold outside them is a single launch.
+SWEEP_RANGES = ((0, 5), (6, 7), (6, 8), (6, 10))
 
 
 def sweep_launches(es, m: int):
@@ -121,9 +122,11 @@ def sweep_launches(es, m: int):
     while e <= top:
         last, klo, khi = e, min(e, m - 1), min(e, m - 1)
         if e <= m - 1:
+            end = min(top, m - 1)
             for lo, hi in SWEEP_RANGES:
-                if lo <= e <= hi and min(hi, top, m - 1) > e:
-                    last, klo, khi = min(hi, top, m - 1), lo, hi
+                if lo <= e <= hi and min(hi, end) > e and (hi >= end or hi in (5, 10)):
+                    last, klo, khi = min(hi, end), lo, hi
+                    break
         out.append((e, last, klo, khi))
         e = last + 1
     return out
@@ -146,13 +149,16 @@ def sweep_bytes_per_pair(m: int, n_written: int, result_byte: bool = False) -> f
 
 
 def pp_sweep_ops_per_pair(m: int, e_lo: int, e_hi: int) -> float:
-    """Integer ops per pair of one per-pair sweep launch (gk_filter_sweep),
-    word formulation: the Hamming mask and the 2K masks of the largest shift
-    count K = min(e_hi, m-1) once (the survey's 9 + 22K per word), and the
-    count (4 per word) for each of the thresholds."""
+    """Logic ops per pair of one per-pair sweep launch (gk_filter_sweep) in
+    the striped form with S words per vector: per word 4 for the Hamming mask
+    (difference 2, dilation, erosion), 5 for each of the 2K shifted masks (the
+    AND with the vacated positions one more) up to the largest shift count K =
+    min(e_hi, m-1), once, and 1 for the count of each threshold.  (The word
+    formulation, 9 + 22K + 4n per word of 32 bases, no longer bounds it.)"""
     W = -(-m // 32)
+    S = 3 if W <= 3 else W if W <= 5 else 8 if W <= 8 else 11
     K = min(e_hi, max(m - 1, 0))
-    return W * (9 + 22 * K + 4 * (e_hi - e_lo + 1))
+    return S * (4 + 10 * K + (e_hi - e_lo + 1))
 
 
 def pp_sweep_bytes_per_pair(m: int, c: float, n_thresholds: int, result_byte: bool = False) -> float:
@@ -545,8 +551,9 @@ def run_mine(args):
             per_e[str(e)] = {"gpairs_s": rate / 1e9, "roofline_gpairs_s": ceil / 1e9, "frac": rate / ceil}
         return {"bound": "alu", "achieved": tops, "peak": ALU_PEAK_TOPS, "unit": "Tops/s",
                 "frac": tops / ALU_PEAK_TOPS, "traffic": recorded_traffic("c2-100bp-e0..10"),
-                "kernel": ("filter_pair2_kernel<W, 4, K> (e 0-2, two pairs per thread, shift count fixed at "
-                           "compile time) | filter_pair2_kernel<W, 2> (e 3-10)"),
+                "kernel": ("filter_pair2_kernel<W, 4, K, -1> (e 0-2, two pairs per thread, shift count fixed at "
+                           "compile time) | filter_pair2_kernel<W, 2, -1, S> (e 3-10: overlapping words, striped "
+                           "from 8)"),
                 "ops_basis": "W*(9 + 22e + 4) per pair (word formulation)", "peak_basis": peak_basis,
                 "bytes_side": {"achieved_gbs": gbs, "peak_gbs": hbm_peak, "frac": gbs / hbm_peak,
                                "bytes_per_pair": bpp},
@@ -639,12 +646,12 @@ def run_mine(args):
         survey_b = w.n_pairs * bytes_per_pair(m, c, False) * n_th
         survey_ops = sum(w.n_pairs * ops_per_pair(m, e) for e in E_SWEEP)
         W = -(-m // 32)
-        kern = f"filter_pair2_kernel<{W}, 3>" if W <= 4 else f"filter_kernel<{W}, 3, false>"
+        kern = f"sweep_pair2_kernel<{W}, S>" if W <= 5 else f"filter_kernel<{W}, 3, false, S>"
         return {"bound": "alu", "achieved": tops, "peak": ALU_PEAK_TOPS, "unit": "Tops/s",
                 "frac": tops / ALU_PEAK_TOPS, "traffic": recorded_traffic("c2-100bp-sweep", kind="per_pair"),
                 "kernel": kern + " (gk_filter_sweep, one launch for every threshold)",
-                "ops_basis": "W*(9 + 22*K + 4*n_thresholds) per pair, K = min(e_hi, m-1): the word formulation's "
-                             "masks once up to the largest threshold, the count per threshold",
+                "ops_basis": "S*(4 + 10*K + n_thresholds) logic ops per pair, S stripes, K = min(e_hi, m-1): the "
+                             "striped form's masks once up to the largest threshold, the count per threshold",
                 "peak_basis": peak_basis, "launch_ms": sweep_ms,
                 "bytes_side": {"achieved_gbs": gbs, "peak_gbs": hbm_peak, "frac": gbs / hbm_peak,
                                "bytes_per_pair": bts / w.n_pairs,

@@ -1435,18 +1435,15 @@ cudaError_t launch_filter_variant(const FilterArgs &a, cudaStream_t stream) {
   if (a.compact == 0) {
     const uint64_t threads = (a.n_pairs + 1) / 2;
     const unsigned grid = (unsigned)((threads + kFilterThreads - 1) / kFilterThreads);
-    // Two pairs per thread for W <= 4 and the striped sweep of W = 5: the
-    // linear form at W = 5 (2 blocks per SM with its registers unspilled)
-    // measured 40% slower at e = 2, 150 bp.
-    if constexpr (VARIANT == 3 && (W <= 4 || S == 5)) {
-      if (a.m > 0) {
-        sweep_pair2_kernel<W, S><<<grid, kFilterThreads, 0, stream>>>(a);
-        return cudaGetLastError();
-      }
-    }
-    if constexpr ((VARIANT == 2 || VARIANT == 4) && (W <= 4 || S == 5)) {
-      if (a.m > 0) {
-        if constexpr (VARIANT == 4) {
+    // Two pairs per thread for W <= 4 and striped at W = 5: the linear form
+    // there (2 blocks per SM with its registers unspilled) measured 40% slower
+    // at e = 2, 150 bp.  W > 1 implies m > 0.
+    constexpr bool kPairs = VARIANT >= 2 && (W <= 4 || S == 5);
+    if constexpr (kPairs) {
+      if (W > 1 || a.m > 0) {
+        if constexpr (VARIANT == 3) {
+          sweep_pair2_kernel<W, S><<<grid, kFilterThreads, 0, stream>>>(a);
+        } else if constexpr (VARIANT == 4) {
           // shift count = the threshold, 0..2, below m (checked by the caller)
           switch (a.fixed_e) {
             case 0: filter_pair2_kernel<W, 4, 0, S><<<grid, kFilterThreads, 0, stream>>>(a); break;
@@ -1460,8 +1457,8 @@ cudaError_t launch_filter_variant(const FilterArgs &a, cudaStream_t stream) {
         return cudaGetLastError();
       }
     }
-    if constexpr (VARIANT == 4) {
-      return cudaErrorInvalidValue;  // VARIANT 4 is the two-pair kernel only
+    if constexpr (VARIANT == 4 || (kPairs && W > 1)) {
+      return cudaErrorInvalidValue;  // the two-pair kernels only
     } else {
       filter_kernel<W, VARIANT, false, S><<<blocks, kFilterThreads, 0, stream>>>(a);
       return cudaGetLastError();
