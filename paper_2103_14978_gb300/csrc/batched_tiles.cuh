@@ -10,7 +10,8 @@
 //                    order.  One launch, no scratch.
 //   large launches   write the tile's pairs as 16-byte records in sorted order
 //                    (plan_kernel); filter launches, one per range of read
-//                    lengths, then take one group of 8 tiles at a time
+//                    lengths or one for all, then take one group of 8 tiles
+//                    at a time
 //                    (groups_kernel).  All blocks of a launch run one group's
 //                    code at about the same time: with 50-300 bp mixed, a
 //                    tile's groups in turn waited for instructions a fifth of
@@ -38,11 +39,22 @@ constexpr int kPlanPer = 8;         // pairs of a plan_kernel thread
 constexpr uint32_t kPlanPairs = kPlanThreads * kPlanPer;  // its tile
 constexpr uint32_t kTilesPairs = 2048;  // pairs of its tile, at most: 36 KB
 
-// Launches above this many pairs go through records.  A launch of one length
-// would filter in its tiles at any size; how many lengths it mixes is not known
-// on the host.
-constexpr uint64_t kTilesFused = 2000000;
-constexpr uint32_t kGroupTiles = 8;  // plan tiles of a work item of groups_kernel
+// Launches of up to this many pairs filter in their tiles.  How many lengths a
+// launch mixes is not known on the host; rows of up to 4 words hold few (8
+// groups).  Measured, in tiles / through records: 50-300 bp, 0.25M pairs 0.123
+// ms / 0.21 (a launch-wide sort), 1M 0.293 / 0.153; 100 bp 1.26M and 150 bp
+// 1.25M, two calls, 0.21 / 0.34.
+template <int WHI>
+constexpr uint64_t tiles_fused() {
+  return WHI <= 4 ? 2000000 : 600000;
+}
+// Up to this many pairs the records of all lengths (of up to 10 words) are
+// filtered by one launch; above, one per range of lengths has more warps in
+// flight for the short ones (4 words: 32 a SM, else 16).  Mixed, 3M pairs: 0.338
+// ms in one, 0.342 in four.
+constexpr uint64_t kTilesOneRange = 8000000;
+constexpr uint32_t kGroupTiles = 8;     // tiles of a work item of groups_kernel
+constexpr uint32_t kSliceRecords = 1024;  // of its slices, at most
 constexpr int kGroupThreads = 128;
 
 // Shared bytes of a tile: read id, offset (later the result), length, key,
@@ -356,20 +368,40 @@ __global__ void __launch_bounds__(kPlanThreads, 2) plan_kernel(const BatchArgs b
 
 // The groups of reads of WLO .. WTOP words out of records planned for reads of
 // at most WHI: persistent blocks take one group of kGroupTiles tiles at a time,
-// all tiles of the longest reads first.
+// all tiles of the longest reads first.  Where a launch is small, or most pairs
+// are of one group (up to 32768 records), these items are too few to go round
+// the SMs, so a group's are cut into slices: of a quarter of a block's share, at
+// most kSliceRecords, as the counts of 32 tiles, evenly spread, suggest (the
+// same tiles for every block).
 template <int WHI, int WLO, int WTOP>
 __global__ void __launch_bounds__(kGroupThreads, WTOP <= 4 ? 8 : (WTOP <= 5 ? 6 : (WTOP <= 10 ? 4 : 2)))
     groups_kernel(const BatchArgs b, uint32_t tiles, const uint32_t *desc, uint32_t *counter) {
-  __shared__ uint32_t s_first[kGroupTiles], s_end[kGroupTiles + 1], s_item;
+  constexpr uint32_t kFirst = 2 * (WHI - WTOP), kCount = 2 * (WTOP - WLO + 1);
+  __shared__ uint32_t s_first[kGroupTiles], s_end[kGroupTiles + 1], s_item, s_slices[kCount];
   const FilterArgs &a = b.f;
   const uint32_t parts = (tiles + kGroupTiles - 1) / kGroupTiles;
-  constexpr uint32_t kFirst = 2 * (WHI - WTOP), kCount = 2 * (WTOP - WLO + 1);
+  for (uint32_t g = threadIdx.x / 32; g < kCount; g += kGroupThreads / 32) {
+    const uint32_t at = (uint32_t)((uint64_t)tiles * (threadIdx.x & 31u) / 32u);
+    const uint32_t count = __reduce_add_sync(0xffffffffu, desc[(uint64_t)(kFirst + g) * tiles + at] >> 16);
+    if ((threadIdx.x & 31u) == 0) s_slices[g] = count;
+  }
+  __syncthreads();
+  if (threadIdx.x < 32) {
+    const uint32_t count = threadIdx.x < kCount ? s_slices[threadIdx.x] : 0u;
+    const uint64_t range = (uint64_t)__reduce_add_sync(0xffffffffu, count) * tiles / 32u;
+    const uint32_t slice = max((uint32_t)kGroupThreads, (uint32_t)min_u64(kSliceRecords, range / (4u * gridDim.x)));
+    if (threadIdx.x < kCount) s_slices[threadIdx.x] = max(1u, count / (32u / kGroupTiles * slice));
+  }
   for (;;) {
     if (threadIdx.x == 0) s_item = atomicAdd(counter, 1u);
     __syncthreads();
-    const uint32_t item = s_item;
-    if (item >= parts * kCount) break;
-    const uint32_t group = kFirst + item / parts, t0 = item % parts * kGroupTiles;
+    uint32_t item = s_item, g = 0, slices = s_slices[0];
+    while (g < kCount && item >= parts * slices) {
+      item -= parts * slices;
+      if (++g < kCount) slices = s_slices[g];
+    }
+    if (g == kCount) break;
+    const uint32_t group = kFirst + g, t0 = item / slices * kGroupTiles, slice = item % slices;
     if (threadIdx.x < 32) {
       const uint32_t lane = threadIdx.x;
       const uint32_t d = lane < kGroupTiles && t0 + lane < tiles ? desc[(uint64_t)group * tiles + t0 + lane] : 0u;
@@ -385,7 +417,9 @@ __global__ void __launch_bounds__(kGroupThreads, WTOP <= 4 ? 8 : (WTOP <= 5 ? 6 
       if (lane == 0) s_end[0] = 0;
     }
     __syncthreads();
-    const uint32_t n = s_end[kGroupTiles];
+    const uint32_t all = s_end[kGroupTiles];
+    const uint32_t per = ((all + slices - 1) / slices + kGroupThreads - 1) / kGroupThreads * kGroupThreads;
+    const uint32_t n = min(all, (slice + 1) * per), j0 = slice * per + threadIdx.x;
     auto record = [&](uint32_t j) -> uint4 {
       uint32_t q = 0;  // the tile that holds record j
 #pragma unroll
@@ -394,8 +428,8 @@ __global__ void __launch_bounds__(kGroupThreads, WTOP <= 4 ? 8 : (WTOP <= 5 ? 6 
       return b.s.rec[(uint64_t)(t0 + q) * kPlanPairs + s_first[q] + (j - s_end[q])];
     };
     // The next pair's record is loaded while this one's words are.
-    uint4 next = threadIdx.x < n ? record(threadIdx.x) : make_uint4(0u, 0u, 0u, 0u);
-    for (uint32_t j = threadIdx.x; j < n; j += kGroupThreads) {
+    uint4 next = j0 < n ? record(j0) : make_uint4(0u, 0u, 0u, 0u);
+    for (uint32_t j = j0; j < n; j += kGroupThreads) {
       const uint4 rec = next;
       if (j + kGroupThreads < n) next = record(j + kGroupThreads);
       const uint32_t e = rec.w & 0xFFFFu;
@@ -416,7 +450,7 @@ cudaError_t launch_groups(const BatchArgs &b, uint32_t tiles, const uint32_t *de
 
 template <int WHI>
 cudaError_t launch_tiles(const BatchArgs &b, cudaStream_t stream) {
-  if (b.f.n_pairs <= kTilesFused) {
+  if (b.f.n_pairs <= tiles_fused<WHI>()) {
     // Small launches take smaller tiles, so that every SM gets several.
     uint32_t tile = kTilesPairs;
     while (tile > (uint32_t)kTilesThreads && b.f.n_pairs / tile < 1216) tile /= 2;
@@ -434,6 +468,12 @@ cudaError_t launch_tiles(const BatchArgs &b, cudaStream_t stream) {
   err = cudaGetLastError();
   if constexpr (WHI > 10)
     if (err == cudaSuccess) err = launch_groups<WHI, 11, WHI>(b, tiles, desc, b.s.counters + 4, n, stream);
+  if constexpr (WHI > 4)
+    if (b.f.n_pairs <= kTilesOneRange) {
+      constexpr int kTop = WHI < 10 ? WHI : 10;
+      if (err == cudaSuccess) err = launch_groups<WHI, 1, kTop>(b, tiles, desc, b.s.counters, n, stream);
+      return err;
+    }
   if constexpr (WHI > 8)
     if (err == cudaSuccess) err = launch_groups<WHI, 9, 10>(b, tiles, desc, b.s.counters + 3, n, stream);
   if constexpr (WHI > 4) {

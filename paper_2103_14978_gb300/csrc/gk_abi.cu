@@ -274,7 +274,7 @@ int gk_filter(gk_ref_t ref, const uint32_t *reads, uint32_t stride_words, uint64
   // reads: the queue wins from e >= 1 at W >= 7 (200-300 bp), from e >= 3 at
   // W = 5 (150 bp) and from e >= 7 at W = 4 (100 bp); below them one thread
   // per pair is faster, its loads issued together.  Per-pair thresholds
-  // always queue.
+  // without the edge OR always queue (with it they sort, filter_by_e_kernel).
   const uint32_t e_queue = W >= 7 ? 1u : (W >= 5 ? 3u : 7u);
   const bool n_dense = (double)ref->n_undefined * (double)m >= 0.05 * (double)ref->n_bases;
   a.compact = (ref->n_undefined > 0 && n_pairs < (1ull << 32) && m > 0 &&

@@ -68,3 +68,15 @@ def test_through_records(lengths):
     want = np.where(ed == O.UNDEFINED, gk.GK_RESULT_UNDEFINED,
                     np.where(ed == O.INVALID, gk.GK_RESULT_INVALID, np.minimum(ed, gk.GK_RESULT_MAX_COUNT)))
     assert (res == want.astype(np.uint8)).all()
+
+
+@pytest.mark.parametrize("lengths", [(150, 150), (250, 250)])
+@pytest.mark.parametrize("n_pairs", [600_001, 2_000_357, 8_004_099])
+def test_records_of_one_length(lengths, n_pairs):
+    """One group holds nearly every pair, so its items are cut into slices; one
+    filter launch up to 8 million pairs, one per range of lengths above."""
+    w = workload(lengths, n_pairs, 4200 + lengths[1])
+    acc, ed, err = run(w)
+    idx = np.concatenate([np.arange(0, w.n_pairs, 211), np.arange(w.n_pairs - 500, w.n_pairs)])
+    assert_same((acc[idx], ed[idx]), oracle_run(w, idx=idx), f"{lengths} n={n_pairs}")
+    assert err == int((ed == O.INVALID).sum())
