@@ -333,7 +333,7 @@ uint64_t gk_filter_batched_workspace(uint64_t n_pairs);
  *               n_pairs) bytes, 256-byte aligned, owned by the caller; its
  *               contents need no initialisation and are garbage afterwards;
  *               two calls in flight at once need two workspaces
- * With words_per_thread 1 enqueues one kernel for a small launch (600 thousand
+ * With words_per_thread 1 enqueues one kernel for a small launch (300 thousand
  * pairs; 2 million with rows of up to 4 words), above that a planning kernel and
  * one filter kernel or one per range of read lengths; else a
  * memset, three planning kernels (classify, scan, scatter) and the persistent

@@ -23,10 +23,10 @@
 // 1.15 of 5.3 ms for 50M pairs.
 //
 // Measured on GB300, 50M pairs of 50-300 bp, per-pair thresholds of 2, 5 and
-// 10%, random order: 5.3 -> 4.7 ms per graph launch (planning
+// 10%, random order: 5.43 -> 4.65 ms per graph launch (planning
 // 0.7, bound by the gathers of read length and N flag; the filters by the ALU
 // pipe, those of up to 128 bp by the gathers of shuffled read rows); a server round of 3M pairs
-// of 100, 150 and 250 bp (three calls) 0.391 -> 0.262 ms.
+// of 100, 150 and 250 bp (three calls) 0.392 -> 0.268 ms.
 #pragma once
 
 #include "batched.cuh"
@@ -42,11 +42,11 @@ constexpr uint32_t kTilesPairs = 2048;  // pairs of its tile, at most: 36 KB
 // Launches of up to this many pairs filter in their tiles.  How many lengths a
 // launch mixes is not known on the host; rows of up to 4 words hold few (8
 // groups).  Measured, in tiles / through records: 50-300 bp, 0.25M pairs 0.123
-// ms / 0.21 (a launch-wide sort), 1M 0.293 / 0.153; 100 bp 1.26M and 150 bp
-// 1.25M, two calls, 0.21 / 0.34.
+// ms / 0.217 (a launch-wide sort), 0.5M 0.222 / not measured, 1M 0.293 / 0.132;
+// 250 bp 1M 0.129 / 0.110.
 template <int WHI>
 constexpr uint64_t tiles_fused() {
-  return WHI <= 4 ? 2000000 : 600000;
+  return WHI <= 4 ? 2000000 : 300000;
 }
 // Up to this many pairs the records of all lengths (of up to 10 words) are
 // filtered by one launch; above, one per range of lengths has more warps in
