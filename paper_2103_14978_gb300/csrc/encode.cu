@@ -44,9 +44,23 @@ encode_reads_kernel(const uint8_t *__restrict__ ascii, uint64_t stride, const ui
     const uint64_t n16 = need / 16;
     const uint4 *s4 = reinterpret_cast<const uint4 *>(src);
     uint4 *t4 = reinterpret_cast<uint4 *>(tile);
-    for (uint64_t i = threadIdx.x; i < n16; i += blockDim.x) t4[i] = s4[i];
+    // Rows of one length that are mostly padding: the padding stays where it is
+    // (500k reads in rows of 512 bytes, of 76 bases 68 -> 34 us, of 160 86 -> 62).
+    const uint32_t row16 = (uint32_t)(stride / 16), len16 = (fixed_len + 15u) / 16u;
+    if (!lens && stride % 16 == 0 && 2 * len16 <= row16) {
+      for (uint32_t i = threadIdx.x; i < (uint32_t)nseq * len16; i += blockDim.x) {
+        const uint32_t at = i / len16 * row16 + i % len16;
+        if (at < n16) t4[at] = s4[at];
+      }
+    } else {
+      // Two loads of a thread in flight (four: 200-320 bases in rows of 512 bytes
+      // 5-9% slower; eight 20-30%).
+#pragma unroll 2
+      for (uint64_t i = threadIdx.x; i < n16; i += blockDim.x) t4[i] = s4[i];
+    }
     for (uint64_t i = n16 * 16 + threadIdx.x; i < need; i += blockDim.x) tile[i] = src[i];
   } else {
+#pragma unroll 4
     for (uint64_t i = threadIdx.x; i < need; i += blockDim.x) tile[i] = src[i];
   }
   __syncthreads();
