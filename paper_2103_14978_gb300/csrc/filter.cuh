@@ -1543,19 +1543,36 @@ cudaError_t launch_filter_variant(const FilterArgs &a, cudaStream_t stream) {
 //   250 bp 4M  e 2 158 / 162, 5 263 / 222, 25 1062 / 660
 //   280 bp 3M  e 6 248 / 267, 14 514 / 496
 //   300 bp 3M  e 6 269 / 279, 15 594 / 533, 30 1136 / 891
+// Striped, every step erodes its masks; linear, each written threshold is
+// eroded and corrected by itself.  So few thresholds at the end of many steps
+// favour the linear form (2M pairs of 64 bp at e = 12..15 79 us, striped 88; of
+// 160 bp at 5..10 138 / 146, at 12..15 168 / 184), and rows counts them.  (One
+// threshold alone is gk_filter's.)  The queue of defined pairs keeps W = 9, 10
+// linear: 11 stripes leave it one block of 256 an SM (2M pairs of 300 bp, 0.1%
+// N, e = 0..10 306 us, striped 383).  At 150 bp and largest shift count 3, pairs
+// of different reads run 5% slower striped, pairs that share theirs 20% faster.
 // W = 1 needs one linear word and three stripes; from W = 11 the stripes spill.
+template <int W, int S>
+__host__ bool sweep_striped(uint32_t K, uint32_t rows, int queue) {
+  if (S == 11) return !queue && K >= (W == 9 ? 14u : 12u) && rows >= 6;
+  if (W == 2) return 3 * rows > K;
+  if (W == 4 && S == 5) return K >= 3 && 3 * rows > K;
+  if (W == 5 && S == 8) return K >= 10 && rows >= 9;
+  if (W == 6) return K >= 9 && rows >= 6;
+  if (W == 7) return K >= 4;
+  if (W == 5) return K >= 3;
+  return (W == 3 && S == 3) || W == 4 || (K >= 3 && K + rows >= 7);
+}
 template <int W>
 cudaError_t launch_sweep(const FilterArgs &a, cudaStream_t stream) {
   if constexpr (W >= 2 && W <= 10) {
     constexpr int S0 = W <= 3 ? 3 : (W <= 5 ? W : (W <= 8 ? 8 : 11));
     constexpr int S1 = W == 3 ? 4 : (W == 4 ? 5 : (W == 5 ? 8 : 0));  // reads S0 does not hold
-    constexpr uint32_t from0 = W <= 4 ? 0 : W == 5 ? 3 : W == 6 ? 9 : W == 7 ? 4 : W == 8 ? 3 : W == 9 ? 14 : 9;
-    constexpr uint32_t from1 = W == 5 ? 10 : 3;
-    const uint32_t K = min(a.sweep_hi, a.m - 1);
+    const uint32_t K = min(a.sweep_hi, a.m - 1), rows = K - min(a.fixed_e, a.m - 1) + 1;
     if (a.m <= stripe_limit<S0>()) {
-      if (K >= from0) return launch_filter_variant<W, 3, S0>(a, stream);
+      if (sweep_striped<W, S0>(K, rows, a.compact)) return launch_filter_variant<W, 3, S0>(a, stream);
     } else if constexpr (S1 > 0) {
-      if (K >= from1) return launch_filter_variant<W, 3, S1>(a, stream);
+      if (sweep_striped<W, S1>(K, rows, a.compact)) return launch_filter_variant<W, 3, S1>(a, stream);
     }
   }
   return launch_filter_variant<W, 3>(a, stream);
@@ -1573,7 +1590,9 @@ cudaError_t launch_sweep(const FilterArgs &a, cudaStream_t stream) {
 // K = 9 279 / 315, 17 477 / 451; of 200 bp K = 7 258 / 267, 10 340 / 311; 4M of
 // 250 bp K = 5 188 / 209, 8 257 / 242, 25 687 / 473; 3M of 280 bp K = 14 345 /
 // 326; of 300 bp K = 9 258 / 258, 15 400 / 347; 128 and 160 bp (S = 5 and 8 with
-// 20 rows) no faster up to K = 16.
+// 20 rows) no faster up to K = 16.  In the queue of defined pairs 11 stripes win
+// from K = 25 (2M pairs of 300 bp, 0.1% N: K = 12 237 / 282 us, 20 341 / 348, 25
+// 401 / 392, 30 467 / 432).
 //
 // Up to shift count 7 in overlapping words where they hold the read (m <= 30 W)
 // and W <= 8, ordinary / overlapping words in us on the same launches: 50 bp K =
@@ -1594,7 +1613,7 @@ cudaError_t launch_single(const FilterArgs &a, cudaStream_t stream) {
     if (single_overlaps<W>(a)) return launch_filter_variant<W, 2, -1>(a, stream);
   if constexpr (W >= 3 && W <= 10) {
     constexpr int S = W <= 5 ? W : (W <= 8 ? 8 : 11);
-    if (a.m <= stripe_limit<S>() && a.fixed_e >= single_striped_from<W>())
+    if (a.m <= stripe_limit<S>() && a.fixed_e >= (S == 11 && a.compact ? 25u : single_striped_from<W>()))
       return launch_filter_variant<W, 2, S>(a, stream);
   }
   return launch_filter_variant<W, 2>(a, stream);

@@ -310,6 +310,12 @@ int gk_filter_sweep(gk_ref_t ref, const uint32_t *reads, uint32_t stride_words, 
   if (count_mode != GK_COUNT_RUNS4 && count_mode != GK_COUNT_POPCOUNT)
     return fail(GK_EINVAL, "gk_filter_sweep: unknown count_mode");
   if (reads && !aligned(reads, 8)) return fail(GK_EINVAL, "gk_filter_sweep: reads must be 8-byte aligned");
+  // One threshold: the launches chosen for it (2M pairs of 160 bp at e = 15: 151 us,
+  // swept 176).  Above 10 words the sweep is the faster one (512 bp at e = 5: 176
+  // us, 186).
+  if (e_lo == e_hi && W <= 10)
+    return gk_filter(ref, reads, stride_words, n_reads, read_nflag, m, pair_read, pair_off, nullptr, e_lo, n_pairs,
+                     count_mode, flags, accept_out, edits_out, err_count, stream);
   gk::FilterArgs a{};
   a.ref_hl = ref->hl;
   a.ref_nidx = ref->nidx;
