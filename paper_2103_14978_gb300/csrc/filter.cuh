@@ -869,6 +869,9 @@ __device__ __forceinline__ void filter_and_write(const FilterArgs &a, uint64_t p
       pair_planes<W>(x, rh, rl, gh[0], gl[0]);
       overlap_counts<W, 1, -1>(a.m, min(a.fixed_e, a.m - 1), a.count_mode, rh, rl, gh, gl, c);
       count = c[0];
+    } else if constexpr (VARIANT == 6) {  // one form per warp
+      count = __any_sync(__activemask(), min(x.e, a.m - 1) > 30) ? filter_loaded<W, false>(a, x)
+                                                                 : filter_loaded_deferred<W>(a, x);
     } else
       count = VARIANT == 4   ? filter_loaded_deferred<W, true>(a, x)
               : VARIANT == 2 ? filter_loaded_deferred<W>(a, x)
@@ -951,7 +954,8 @@ constexpr size_t compact_smem_bytes() {
 // 2: edge OR on and one threshold in 2..30, deferred erosion; 3: edge OR on,
 // a sweep of thresholds up to 30 (sweep_and_write).  2 and 3 are striped in S
 // words (S > 0), 2 and 4 in overlapping words (S = -1, shift counts up to
-// kOverlapMax) or linear (S = 0).
+// kOverlapMax) or linear (S = 0).  6: edge OR on, per-pair thresholds in pair
+// order, deferred erosion where a warp's shift counts allow it.
 //
 // COMPACT false: one thread per pair.  COMPACT true (inputs with many
 // undefined pairs): persistent warps take 32 pairs at a time (their ids
@@ -1309,38 +1313,90 @@ __global__ void __launch_bounds__(kFilterThreads, S == 5 ? 6 : 8) sweep_pair2_ke
   }
 }
 
+// Classes of shift counts that a tile of pairs is sorted by: each K up to 30
+// (deferred erosion) its own, above that steps that widen with K (31..62 by 2,
+// 63..126 by 8, then by 16: at most an eighth of K, so that a warp's pairs still
+// take about the same number of exact steps).
+constexpr uint32_t kShiftClasses = 64, kExactClass = 31;  // kExactClass: K = 31, 32
+__host__ __device__ __forceinline__ uint32_t shift_class(uint32_t K) {  // K <= 255
+  return K <= 30 ? K : (K <= 62 ? 31u + (K - 31u) / 2u : (K <= 126 ? 47u + (K - 63u) / 8u : 55u + (K - 127u) / 16u));
+}
+
+// A counting sort's rank of each lane's class among the equal ones before it
+// (class none: no rank), one counter update per class and warp.
+__device__ __forceinline__ uint32_t class_rank(uint32_t cls, uint32_t none, uint32_t *s_n) {
+  const uint32_t lane = threadIdx.x & 31u;
+  const unsigned peers = __match_any_sync(0xffffffffu, cls);
+  const int leader = __ffs(peers) - 1;
+  uint32_t at = 0;
+  if (cls != none && (int)lane == leader) at = atomicAdd(&s_n[cls], (unsigned)__popc(peers));
+  return __shfl_sync(0xffffffffu, at, leader) + __popc(peers & ((1u << lane) - 1u));
+}
+
+// Counts per class into each class's first slot, the largest first (one warp,
+// two classes per lane); returns the slots used in lane 31.
+__device__ __forceinline__ uint32_t class_starts(uint32_t *s_n) {
+  const uint32_t lane = threadIdx.x & 31u, c = kShiftClasses - 1u - 2u * lane;
+  const uint32_t n0 = s_n[c], n1 = s_n[c - 1];
+  uint32_t v = n0 + n1;
+  for (int d = 1; d < 32; d <<= 1) {
+    const uint32_t o = __shfl_up_sync(0xffffffffu, v, d);
+    if (lane >= (uint32_t)d) v += o;
+  }
+  s_n[c] = v - n0 - n1;
+  s_n[c - 1] = v - n1;
+  return v;
+}
+
 // Per-pair thresholds with the edge OR on, one read length.  In pair order a
-// warp takes as many shift steps as its largest threshold asks for, all with
-// exact erosion (a pair's threshold may be any).  Here a block takes a tile of
-// pairs, writes the trivial outcomes, and sorts the others by shift count in
-// shared memory (a counting sort over K = 0 .. 30 and one class for more), so
-// that a warp's pairs need about the same number of steps, of the deferred
-// form (striped in S words; S = 0: linear) up to 30 and exact above.  Results
-// are staged in shared memory and written in pair order.  A genome's undefined
-// pairs drop out with the sort, so N-dense inputs need no queue.
+// warp takes as many shift steps as its largest threshold asks for.  Here a
+// block takes a tile of pairs, writes the trivial outcomes, and sorts the
+// others by shift count in shared memory (a counting sort over shift_class),
+// so that a warp's pairs need about the same number of steps, of the deferred
+// form (striped in S words where shift counts reach FROM; S = 0: linear) up to
+// 30 and exact above.  Results are staged in shared memory and written in pair
+// order.  A genome's undefined pairs drop out with the sort, so N-dense inputs
+// need no queue.
 //
-// Measured on GB300, 10M pairs of 150 bp, thresholds 3, 8 and 15 mixed: 1071 ->
-// 423 us.
+// A tile keeps its order where the sort would cost more than it saves
+// (worth_sorting).  It saves half the spread of the shift counts (a warp takes
+// its largest) and, for lanes idle on settled pairs, their share of a pair's
+// steps; it costs about two shift steps per pair in tiles of 512, half that in
+// tiles of 1024, twice that in smaller ones, and twice again above 10 words,
+// whose rows it gathers out of order.  The largest tiles are nearly always worth
+// it and rank their pairs while the next batch loads.
+//
+// Measured on GB300, one pair per thread with exact erosion / always sorted and
+// striped / here: 10M pairs of 150 bp, thresholds 3, 8 and 15 mixed 1112 / 441 /
+// 446 us; 2M pairs with thresholds 0..2 of 100 bp 47 / 62 / 46, with threshold 2
+// of 170 bp 62 / 109 / 57, of 300 bp 107 / 150 / 88; with thresholds 0..255 of 300
+// bp 6180 / 6098 / 3542 (one class above 30 before).
 constexpr int kTilePairs = 1024;  // pairs of a tile, at most
 
-template <int W, int S>
-__global__ void __launch_bounds__(kFilterThreads, S > 0 ? MinBlocks<W, false, S>::value : MinBlocks<W, true>::value * 2)
+template <int W, int S, int FROM, int TILE>
+__global__ void __launch_bounds__(kFilterThreads, S > 0 ? MinBlocks<W, false, S>::value : (W <= 2 ? 10 : (W <= 4 ? 8 : MinBlocks<W, true>::value * 2)))
     filter_by_e_kernel(const FilterArgs a, uint32_t tile) {
-  constexpr int kClasses = 32, kBatch = 4;
-  __shared__ uint32_t s_rid[kTilePairs], s_off[kTilePairs];
-  __shared__ uint16_t s_at[kTilePairs], s_edits[kTilePairs];
-  __shared__ uint8_t s_e[kTilePairs], s_class[kTilePairs], s_accept[kTilePairs];
-  __shared__ uint32_t s_n[kClasses], s_first[kClasses + 1];
+  // Batches of two pairs where a thread may have no more.
+  constexpr bool kEarly = TILE == kTilePairs;
+  constexpr int kBatch = kEarly ? 4 : 2, kPer = TILE / kFilterThreads;
+  constexpr uint8_t kSettled = 0xff;
+  __shared__ uint32_t s_rid[TILE], s_off[TILE];
+  __shared__ uint16_t s_at[TILE], s_edits[TILE];
+  __shared__ uint8_t s_e[TILE], s_class[TILE], s_accept[TILE], s_class_of[256];
+  __shared__ uint32_t s_n[kShiftClasses], s_range[kFilterWarps], s_used, s_plan;
   const int lane = threadIdx.x & 31;
   const uint64_t base = blockIdx.x * (uint64_t)tile;
   const uint32_t n_here = (uint32_t)min_u64(tile, a.n_pairs - base);
-  if (threadIdx.x < kClasses) s_n[threadIdx.x] = 0;
+  if (threadIdx.x < kShiftClasses) s_n[threadIdx.x] = 0;
+#pragma unroll
+  for (int k = 0; k < 256; k += kFilterThreads) s_class_of[k + threadIdx.x] = (uint8_t)shift_class(k + threadIdx.x);
   __syncthreads();
 
-  // Classify, a batch of pairs per thread at a time: ids, then what they point to.
-  constexpr int kPer = kTilePairs / kFilterThreads;
+  // Classify and, kEarly, rank, a batch of pairs per thread at a time: ids, then
+  // what they point to.
   uint32_t rid[kPer], off[kPer], rank[kPer];
   uint8_t e[kPer], cls[kPer];
+  uint32_t low = kSettled, high = 0, settled = 0;  // this thread's classes; pairs without one
 #pragma unroll
   for (int r0 = 0; r0 < kPer; r0 += kBatch) {
     if (r0 * kFilterThreads >= (int)tile) break;
@@ -1382,61 +1438,104 @@ __global__ void __launch_bounds__(kFilterThreads, S > 0 ? MinBlocks<W, false, S>
         const unsigned bad = __ballot_sync(0xffffffffu, active && status == 2);
         if (bad && lane == 0) atomicAdd(a.err_count, (unsigned)__popc(bad));
       }
-      cls[r] = 0xff;
+      cls[r] = kSettled;
       if (active && status != 0) {
         s_accept[i] = status != 2;
         s_edits[i] = status == 1 ? GK_EDITS_UNDEFINED : GK_EDITS_INVALID;
+        ++settled;
       }
-      if (active && status == 0) cls[r] = (uint8_t)min(min((uint32_t)e[r], a.m - 1), (uint32_t)kClasses - 1);
-      // One counter update per class and warp.
-      const unsigned peers = __match_any_sync(0xffffffffu, cls[r]);
-      const int leader = __ffs(peers) - 1;
-      uint32_t at = 0;
-      if (cls[r] != 0xff && lane == leader) at = atomicAdd(&s_n[cls[r]], (unsigned)__popc(peers));
-      rank[r] = __shfl_sync(0xffffffffu, at, leader) + __popc(peers & ((1u << lane) - 1u));
+      if (active && status == 0) {
+        cls[r] = s_class_of[min((uint32_t)e[r], a.m - 1)];
+        low = min(low, (uint32_t)cls[r]);
+        high = max(high, (uint32_t)cls[r]);
+      }
+      if (kEarly) rank[r] = class_rank(cls[r], kSettled, s_n);
     }
   }
-  __syncthreads();
-  if (threadIdx.x < 32) {  // exclusive scan, most steps first
-    const int c = kClasses - 1 - (int)threadIdx.x;
-    uint32_t v = s_n[c];
-    for (int d = 1; d < 32; d <<= 1) {
-      const uint32_t o = __shfl_up_sync(0xffffffffu, v, d);
-      if (lane >= d) v += o;
+  auto worth_sorting = [&]() {
+    const uint32_t saves = (7 * n_here * (high - low) + 10 * settled * (high + 1)) * (max(tile, 256u) / 256u);
+    return low < kSettled && saves > (W <= 10 ? 48u : 96u) * n_here;
+  };
+  bool sorted = true;
+  if (!kEarly) {
+    low = __reduce_min_sync(0xffffffffu, low);
+    high = __reduce_max_sync(0xffffffffu, high);
+    settled = __reduce_add_sync(0xffffffffu, settled);
+    if (lane == 0) s_range[threadIdx.x / 32] = low | (high << 8) | (settled << 16);
+    __syncthreads();
+    low = kSettled;
+    high = settled = 0;
+#pragma unroll
+    for (int w = 0; w < kFilterWarps; ++w) {
+      const uint32_t v = s_range[w];
+      low = min(low, v & 0xFFu);
+      high = max(high, (v >> 8) & 0xFFu);
+      settled += v >> 16;
     }
-    s_first[c] = v - s_n[c];
-    if (threadIdx.x == 31) s_first[kClasses] = v;
+    sorted = worth_sorting();
+    if (sorted) {
+#pragma unroll
+      for (int r = 0; r < kPer; ++r) {
+        if (r * kFilterThreads >= (int)tile) break;
+        rank[r] = class_rank(cls[r], kSettled, s_n);
+      }
+    }
   }
-  __syncthreads();
+  if (kEarly || sorted) {
+    __syncthreads();
+    if (threadIdx.x < 32) {
+      // kEarly: the counts say how far the classes reach.
+      const uint32_t c = kShiftClasses - 1u - 2u * (uint32_t)lane, n0 = s_n[c], n1 = s_n[c - 1];
+      const unsigned any = __ballot_sync(0xffffffffu, (n0 | n1) != 0);
+      high = __shfl_sync(0xffffffffu, n0 ? c : c - 1, any ? __ffs(any) - 1 : 0);
+      low = any ? __shfl_sync(0xffffffffu, n1 ? c - 1 : c, 31 - __clz(any)) : kSettled;
+      const uint32_t used = __shfl_sync(0xffffffffu, class_starts(s_n), 31);
+      settled = n_here - used;
+      if (lane == 0) {
+        s_used = used;
+        s_plan = high | (worth_sorting() ? 0x100u : 0u);
+      }
+    }
+    __syncthreads();
+    high = s_plan & 0xFFu;
+    sorted = s_plan >= 0x100u;
+  }
 #pragma unroll
   for (int r = 0; r < kPer; ++r) {
     if (r * kFilterThreads >= (int)tile) break;
-    if (cls[r] == 0xff) continue;
-    const uint32_t s = s_first[cls[r]] + rank[r];
+    const uint32_t i = (uint32_t)r * kFilterThreads + threadIdx.x;
+    if (sorted && cls[r] == kSettled) continue;
+    const uint32_t s = sorted ? s_n[cls[r]] + rank[r] : i;
     s_rid[s] = rid[r];
     s_off[s] = off[r];
     s_e[s] = e[r];
     s_class[s] = cls[r];
-    s_at[s] = (uint16_t)((uint32_t)r * kFilterThreads + threadIdx.x);
+    s_at[s] = (uint16_t)i;
   }
-  __syncthreads();
-  const uint32_t n_list = s_first[kClasses];
+  if (sorted) __syncthreads();  // in order a thread reads the entries that it wrote
+  const uint32_t n_list = sorted ? s_used : n_here;
 #pragma unroll 1
   for (uint32_t s = threadIdx.x; s < n_list; s += kFilterThreads) {
+    const uint32_t cl = s_class[s];
+    if (cl == kSettled) continue;
     PairData<W> x;
     x.rid = s_rid[s];
     x.off = s_off[s];
     x.e = s_e[s];
     x.m = a.m;
-    const uint32_t K = s_class[s];
     const uint2 *rp = a.reads + (uint64_t)x.rid * a.stride_words;
 #pragma unroll
     for (int w = 0; w < W; ++w) x.r[w] = rp[w];
     load_window<W, false>(a, x);
     uint32_t count;
-    if (K < kClasses - 1) {
+    if (cl < kExactClass) {
       if constexpr (S > 0)
-        count = filter_loaded_striped<W, S>(a, x, K);
+        // One form per tile: both forms' code does not fit the instruction cache
+        // beside the exact one's; at W = 5 one per warp (one on both sides of
+        // FROM runs striped).
+        count = (W != 5 ? high >= (uint32_t)FROM : __any_sync(__activemask(), cl >= (uint32_t)FROM))
+                    ? filter_loaded_striped<W, S>(a, x, cl)
+                    : filter_loaded_deferred<W>(a, x);
       else
         count = filter_loaded_deferred<W>(a, x);
     } else {
@@ -1446,7 +1545,7 @@ __global__ void __launch_bounds__(kFilterThreads, S > 0 ? MinBlocks<W, false, S>
     s_accept[i] = count <= x.e;
     s_edits[i] = (uint16_t)count;
   }
-  __syncthreads();
+  if (sorted) __syncthreads();
   for (uint32_t i = threadIdx.x; i < n_here; i += kFilterThreads) {
     a.accept[base + i] = s_accept[i];
     a.edits[base + i] = s_edits[i];
@@ -1463,7 +1562,7 @@ cudaError_t launch_filter_variant(const FilterArgs &a, cudaStream_t stream) {
     // Two pairs per thread for W <= 4 and striped at W = 5: the linear form
     // there (2 blocks per SM with its registers unspilled) measured 40% slower
     // at e = 2, 150 bp.  W > 1 implies m > 0.
-    constexpr bool kPairs = VARIANT >= 2 && (W <= 4 || S == 5);
+    constexpr bool kPairs = VARIANT >= 2 && VARIANT <= 4 && (W <= 4 || S == 5);
     if constexpr (kPairs) {
       if (W > 1 || a.m > 0) {
         if constexpr (VARIANT == 3) {
@@ -1630,21 +1729,25 @@ cudaError_t launch_small(const FilterArgs &a, cudaStream_t stream) {
 
 // Launches per-pair thresholds (edge OR on, m > 0).  Tiles shrink with the
 // launch, so that a small one still spreads over the chip.
-template <int W, int S>
+template <int W, int S, int FROM>
 cudaError_t launch_by_e_striped(const FilterArgs &a, cudaStream_t stream) {
   uint32_t tile = kTilePairs;
-  while (tile > (uint32_t)kFilterThreads && a.n_pairs / tile < 4096) tile /= 2;
+  while (tile > (uint32_t)kFilterThreads && a.n_pairs / tile < 2048) tile /= 2;
   const uint64_t blocks = (a.n_pairs + tile - 1) / tile;
-  filter_by_e_kernel<W, S><<<(unsigned)blocks, kFilterThreads, 0, stream>>>(a, tile);
+  if (tile == (uint32_t)kTilePairs)
+    filter_by_e_kernel<W, S, FROM, kTilePairs><<<(unsigned)blocks, kFilterThreads, 0, stream>>>(a, tile);
+  else
+    filter_by_e_kernel<W, S, FROM, kTilePairs / 2><<<(unsigned)blocks, kFilterThreads, 0, stream>>>(a, tile);
   return cudaGetLastError();
 }
 template <int W>
 cudaError_t launch_by_e(const FilterArgs &a, cudaStream_t stream) {
-  if constexpr (W >= 4 && W <= 10) {
+  // W = 6 linear: with both forms registers hold 4 blocks an SM, without 6.
+  if constexpr (W >= 4 && W <= 10 && W != 6) {
     constexpr int S = W <= 5 ? W : (W <= 8 ? 8 : 11);
-    if (a.m <= stripe_limit<S>()) return launch_by_e_striped<W, S>(a, stream);
+    if (a.m <= stripe_limit<S>()) return launch_by_e_striped<W, S, single_striped_from<W>()>(a, stream);
   }
-  return launch_by_e_striped<W, 0>(a, stream);
+  return launch_by_e_striped<W, 0, 0>(a, stream);
 }
 
 }  // namespace gk

@@ -37,12 +37,17 @@ int cuda_check(cudaError_t err, const char *what) {
   return fail(GK_ECUDA, std::string(what) + ": " + cudaGetErrorString(err));
 }
 
-// Variant of the per-pair code for a launch: 5 per-pair thresholds (gk_filter
-// with the edge OR), 4 a threshold 0..2 at W <= 4, 3 a sweep, 2 deferred
-// erosion, 1 exact with every shift below 32, 0 exact for any thresholds.
+// Variant of the per-pair code for a launch: 5 and 6 per-pair thresholds
+// (gk_filter with the edge OR), sorted and in pair order, 4 a threshold 0..2 at
+// W <= 4, 3 a sweep, 2 deferred erosion, 1 exact with every shift below 32, 0
+// exact for any thresholds.
 int filter_variant(const FilterArgs &a, bool pair_k) {
   if (a.out_stride != 0) return 3;  // a threshold sweep (gk_filter_sweep)
-  if (pair_k && a.pair_e && a.edge_on && a.m > 0) return 5;  // sorted by threshold (filter_by_e_kernel)
+  // Sorted by threshold (filter_by_e_kernel).  Reads of at most 64 bases filter
+  // in less time than the sort takes, below 4 million pairs (2M pairs of 50 bp:
+  // thresholds 1, 3 and 5 45 us sorted, 41 in order; threshold 2 41 and 30); of at
+  // most 32, at any size.
+  if (pair_k && a.pair_e && a.edge_on && a.m > 32) return a.m > 64 || a.n_pairs >= 4000000 ? 5 : 6;
   // One threshold 0..2 below m, reads of at most 128 bases, no compaction:
   // the two-pairs-per-thread deferred kernel with the shift count fixed at
   // compile time (measured on GB300 at 100 bp against the exact one-pair
@@ -274,11 +279,12 @@ int gk_filter(gk_ref_t ref, const uint32_t *reads, uint32_t stride_words, uint64
   // reads: the queue wins from e >= 1 at W >= 7 (200-300 bp), from e >= 3 at
   // W = 5 (150 bp) and from e >= 7 at W = 4 (100 bp); below them one thread
   // per pair is faster, its loads issued together.  Per-pair thresholds
-  // without the edge OR always queue (with it they sort, filter_by_e_kernel).
+  // queue without the edge OR and for reads of one word; otherwise they sort or
+  // keep their order (filter_variant).
   const uint32_t e_queue = W >= 7 ? 1u : (W >= 5 ? 3u : 7u);
   const bool n_dense = (double)ref->n_undefined * (double)m >= 0.05 * (double)ref->n_bases;
   a.compact = (ref->n_undefined > 0 && n_pairs < (1ull << 32) && m > 0 &&
-               (pair_e || (n_dense && fixed_e >= e_queue))) ? 1 : 0;
+               (pair_e ? !a.edge_on || W == 1 : n_dense && fixed_e >= e_queue)) ? 1 : 0;
   return gk::cuda_check(gk::launch_filter((int)W, a, (cudaStream_t)stream), "gk_filter: launch");
 }
 
