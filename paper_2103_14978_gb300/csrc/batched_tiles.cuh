@@ -37,7 +37,7 @@ constexpr int kTilesThreads = 256;  // of tiles_kernel
 constexpr int kPlanThreads = 512;   // of plan_kernel
 constexpr int kPlanPer = 8;         // pairs of a plan_kernel thread
 constexpr uint32_t kPlanPairs = kPlanThreads * kPlanPer;  // its tile
-constexpr uint32_t kTilesPairs = 2048;  // pairs of its tile, at most: 36 KB
+constexpr uint32_t kTilesPairs = 1024;  // pairs of tiles_kernel's tile, at most
 
 // Launches of up to this many pairs filter in their tiles.  How many lengths a
 // launch mixes is not known on the host; rows of up to 4 words hold few (8
@@ -225,7 +225,7 @@ __device__ __forceinline__ uint32_t tiles_scan(uint32_t *s_n, int groups) {
 template <int WHI>
 __device__ __forceinline__ void tile_sort(const BatchArgs &b, uint32_t tile, const TileArrays &t, uint32_t *s_n,
                                           uint32_t *slots) {
-  constexpr int kGroups = 2 * WHI, kBatch = 4;
+  constexpr int kGroups = 2 * WHI, kBatch = kTilesPairs / kTilesThreads;
   const FilterArgs &a = b.f;
   const int lane = threadIdx.x & 31;
   const uint64_t base = blockIdx.x * (uint64_t)tile;
@@ -233,34 +233,32 @@ __device__ __forceinline__ void tile_sort(const BatchArgs &b, uint32_t tile, con
   for (int i = threadIdx.x; i < kGroups * 32; i += kTilesThreads) s_n[i] = 0;
   for (uint32_t i = threadIdx.x; i < tile + kGroups * 32; i += kTilesThreads) t.list[i] = kNoSlot;
   __syncthreads();
-  for (uint32_t i0 = 0; i0 < n_here; i0 += kBatch * kTilesThreads) {
-    PairBatch<kBatch, kTilesThreads> x;
-    x.load(b, base + i0, base + n_here);
+  PairBatch<kBatch, kTilesThreads> x;
+  x.load(b, base, base + n_here);
 #pragma unroll
-    for (int r = 0; r < kBatch; ++r) {
-      const uint32_t i = i0 + (uint32_t)r * kTilesThreads + threadIdx.x;
-      const bool active = i < n_here;
-      const int status = x.status(a, r);
-      if (a.err_count) {
-        const unsigned bad = __ballot_sync(0xffffffffu, active && status == 2);
-        if (bad && lane == 0) atomicAdd(a.err_count, (unsigned)__popc(bad));
-      }
-      if (!active) continue;
-      uint32_t key = kNoSlot;
-      if (status == 0) {
-        key = tiles_key<WHI>(a, x.m[r], x.e[r]);
-        atomicAdd(&s_n[key], 1u);
-        t.rid[i] = x.rid[r];
-        t.off[i] = x.off[r];
-        t.m[i] = (uint16_t)x.m[r];
-        t.e[i] = (uint8_t)x.e[r];
-      } else if (a.result_byte) {
-        t.off[i] = (status == 1 ? GK_RESULT_UNDEFINED : status == 2 ? GK_RESULT_INVALID : 0u) << 16;
-      } else {
-        t.off[i] = status == 1 ? (0x10000u | GK_EDITS_UNDEFINED) : status == 2 ? GK_EDITS_INVALID : 0x10000u;
-      }
-      t.key[i] = (uint16_t)key;
+  for (int r = 0; r < kBatch; ++r) {
+    const uint32_t i = (uint32_t)r * kTilesThreads + threadIdx.x;
+    const bool active = i < n_here;
+    const int status = x.status(a, r);
+    if (a.err_count) {
+      const unsigned bad = __ballot_sync(0xffffffffu, active && status == 2);
+      if (bad && lane == 0) atomicAdd(a.err_count, (unsigned)__popc(bad));
     }
+    if (!active) continue;
+    uint32_t key = kNoSlot;
+    if (status == 0) {
+      key = tiles_key<WHI>(a, x.m[r], x.e[r]);
+      atomicAdd(&s_n[key], 1u);
+      t.rid[i] = x.rid[r];
+      t.off[i] = x.off[r];
+      t.m[i] = (uint16_t)x.m[r];
+      t.e[i] = (uint8_t)x.e[r];
+    } else if (a.result_byte) {
+      t.off[i] = (status == 1 ? GK_RESULT_UNDEFINED : status == 2 ? GK_RESULT_INVALID : 0u) << 16;
+    } else {
+      t.off[i] = status == 1 ? (0x10000u | GK_EDITS_UNDEFINED) : status == 2 ? GK_EDITS_INVALID : 0x10000u;
+    }
+    t.key[i] = (uint16_t)key;
   }
   __syncthreads();
   if (threadIdx.x < 32) {
@@ -275,9 +273,13 @@ __device__ __forceinline__ void tile_sort(const BatchArgs &b, uint32_t tile, con
   __syncthreads();
 }
 
+// Resident blocks of tiles_kernel per SM.
+template <int WHI>
+constexpr int kTilesBlocks = WHI <= 4 ? 4 : (WHI <= 10 ? 2 : 1);
+
 // Reads of at most WHI words (the row stride bounds them): sorted and filtered.
 template <int WHI>
-__global__ void __launch_bounds__(kTilesThreads, WHI <= 4 ? 4 : (WHI <= 10 ? 2 : 1))
+__global__ void __launch_bounds__(kTilesThreads, kTilesBlocks<WHI>)
     tiles_kernel(const BatchArgs b, uint32_t tile) {
   extern __shared__ uint32_t s_mem[];
   __shared__ uint32_t s_n[2 * WHI * 32], s_slots, s_next;
@@ -450,18 +452,21 @@ cudaError_t launch_groups(const BatchArgs &b, uint32_t tiles, const uint32_t *de
 
 template <int WHI>
 cudaError_t launch_tiles(const BatchArgs &b, cudaStream_t stream) {
-  if (b.f.n_pairs <= tiles_fused<WHI>()) {
-    // Small launches take smaller tiles, so that every SM gets several.
-    uint32_t tile = kTilesPairs;
-    while (tile > (uint32_t)kTilesThreads && b.f.n_pairs / tile < 1216) tile /= 2;
-    tiles_kernel<WHI><<<(unsigned)((b.f.n_pairs + tile - 1) / tile), kTilesThreads, tiles_smem<WHI>(tile), stream>>>(
-        b, tile);
-    return cudaGetLastError();
-  }
   int dev = 0, sms = 0;
   cudaError_t err = cudaGetDevice(&dev);
   if (err == cudaSuccess) err = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   if (err != cudaSuccess) return err;
+  if (b.f.n_pairs <= tiles_fused<WHI>()) {
+    // The smallest tile whose blocks all run at once: larger ones fill their
+    // groups' warps, but leave SMs without a block.  50-300 bp mixed, 300k pairs:
+    // tiles of 256 128 us, of 1024 60; 250 bp 300k 53 / 36; 36-512 bp 300k 871 / 310;
+    // 150 bp 50k 11 us, of 1024 16.
+    uint32_t tile = kTilesThreads;
+    while (tile < kTilesPairs && b.f.n_pairs > (uint64_t)tile * (uint32_t)sms * kTilesBlocks<WHI>) tile *= 2;
+    tiles_kernel<WHI><<<(unsigned)((b.f.n_pairs + tile - 1) / tile), kTilesThreads, tiles_smem<WHI>(tile), stream>>>(
+        b, tile);
+    return cudaGetLastError();
+  }
   const uint32_t tiles = (uint32_t)((b.f.n_pairs + kPlanPairs - 1) / kPlanPairs), n = (uint32_t)sms;
   uint32_t *desc = b.s.km;  // 2 WHI <= 32 words per 4096 pairs, out of a word per pair
   plan_kernel<WHI><<<tiles, kPlanThreads, 0, stream>>>(b, desc);
