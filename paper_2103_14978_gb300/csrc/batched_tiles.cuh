@@ -126,7 +126,7 @@ __device__ __forceinline__ uint32_t tiles_count(const FilterArgs &a, uint32_t gr
         return c[0];
       }
     }
-    if (a.edge_on && K <= 30) return filter_loaded_deferred<W>(a, x);
+    if (K <= 30) return a.edge_on ? filter_loaded_deferred<W>(a, x) : filter_loaded<W, true>(a, x);
     return filter_loaded<W, false>(a, x);
   }
   if constexpr (W > WLO)
