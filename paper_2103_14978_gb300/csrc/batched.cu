@@ -219,7 +219,7 @@ cudaError_t launch_persistent_wpt8(const BatchArgs &a, uint32_t grid, uint32_t w
 cudaError_t launch_batched(int wpt, const BatchArgs &a, uint32_t blocks_per_sm, uint32_t warps_per_block,
                            cudaStream_t stream) {
   if (a.f.n_pairs == 0) return cudaSuccess;
-  if (wpt == 1) {  // one pair per lane: sorted in tiles, one launch
+  if (wpt == 1) {  // one pair per lane: sorted in tiles (batched_tiles.cuh)
     const uint32_t sw = a.f.stride_words;
     return sw <= 4 ? launch_tiles_w4(a, stream) : sw <= 8 ? launch_tiles_w8(a, stream)
            : sw <= 10 ? launch_tiles_w10(a, stream) : launch_tiles_w16(a, stream);

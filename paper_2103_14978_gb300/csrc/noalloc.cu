@@ -99,8 +99,8 @@ extern "C" int gk_filter_batched_noalloc(gk_ref_t ref, const uint32_t *reads, ui
   void *scratch = nullptr;
   const int rc = scratch_address(&scratch);
   if (rc != GK_OK) return rc;
-  // The pipeline clears what must start at zero on every call (the key
-  // histogram by a memset, the tile counter in its scan kernel) and writes
+  // The pipeline clears what must start at zero on every call (the item counters
+  // in its first kernel; for lane groups the key histogram by a memset) and writes
   // every other scratch word before reading it, so a previous call's contents
   // do no harm.
   return gk_filter_batched(ref, reads, stride_words, n_reads, read_len, read_nflag, pair_read, pair_off, pair_e,
