@@ -1,8 +1,9 @@
-"""Batched filtering of mixed-length pairs: one persistent launch, captured in
-a CUDA graph, with a tiling picked by an autotuner.
+"""Batched filtering of mixed-length pairs: one library call, captured in a
+CUDA graph, with a tiling picked by an autotuner.
 
-The library does all the work (gk_filter_batched: classify, scan, scatter,
-persistent filter).  This module owns the device buffers (workspace,
+The library does all the work (gk_filter_batched: a whole pair per lane, sorted
+and filtered in tiles or through records; or a pair spread over lanes, classify,
+scan, scatter, persistent filter).  This module owns the device buffers (workspace,
 outputs), captures the call into a CUDA graph for replay, and searches the
 tiling space on a sample of the workload, timing each candidate with CUDA
 events.  The autotuner's table is JSON keyed by GPU name and workload
@@ -98,8 +99,9 @@ def _time(bf: BatchedFilter, reps: int) -> float:
 def autotune(ref, reads, stride_words, n_reads, read_len, read_nflag, pair_read, pair_off, pair_e,
              reps: int = 3, budget_s: float = 60.0, log=None):
     """Coordinate search over the tiling on the given (sample) pairs: words
-    per lane first, then tile size, then grid shape; every candidate timed with
-    CUDA events, invalid ones (a block that does not fit) skipped.  The
+    per lane first, then, for a pair spread over lanes, tile size and grid shape
+    (a whole pair per lane does not use them); every candidate timed with CUDA
+    events, invalid ones (a block that does not fit) skipped.  The
     default tiling is always measured; the budget stops the search after it.
     Returns (best tiling tuple, {candidate: ms})."""
     t0 = time.perf_counter()
@@ -127,6 +129,8 @@ def autotune(ref, reads, stride_words, n_reads, read_len, read_nflag, pair_read,
         cand = (wpt,) + best[1:]
         if measure(cand) < results[best]:
             best = cand
+    if best[0] == 1:
+        return best, results
     for tile in TILE_CHOICES:
         cand = (best[0], tile) + best[2:]
         if measure(cand) < results[best]:
