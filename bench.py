@@ -148,17 +148,62 @@ def sweep_bytes_per_pair(m: int, n_written: int, result_byte: bool = False) -> f
     return m / 2 + 8 / 32 + (1 if result_byte else 3) * n_written
 
 
-def pp_sweep_ops_per_pair(m: int, e_lo: int, e_hi: int) -> float:
-    """Logic ops per pair of one per-pair sweep launch (gk_filter_sweep) in
-    the striped form with S words per vector: per word 4 for the Hamming mask
-    (difference 2, dilation, erosion), 5 for each of the 2K shifted masks (the
-    AND with the vacated positions one more) up to the largest shift count K =
-    min(e_hi, m-1), once, and 1 for the count of each threshold.  (The word
-    formulation, 9 + 22K + 4n per word of 32 bases, no longer bounds it.)"""
+def stripes_of(m: int) -> int:
+    """Words per vector of the striped form for a read of m bases (0: none): the
+    smallest of 3, 4, 5, 8 and, above 8 words, 11 that is at least ceil(m/32) and
+    holds m + 2 (even) or m + 4 (odd) positions."""
     W = -(-m // 32)
-    S = 3 if W <= 3 else W if W <= 5 else 8 if W <= 8 else 11
+    fit = [S for S in ((3, 4, 5, 8) if W <= 8 else (11,)) if S >= W and m <= 32 * S - (4 if S & 1 else 2)]
+    return fit[0] if fit and W >= 2 else 0
+
+
+def pp_sweep_ops_per_pair(m: int, e_lo: int, e_hi: int) -> float:
+    """Logic ops per pair of one per-pair sweep launch (gk_filter_sweep) of many
+    thresholds: in the striped form with S words per vector, per word 4 for the
+    Hamming mask (difference 2, dilation, erosion), 5 for each of the 2K
+    shifted masks (the AND with the vacated positions one more) up to the
+    largest shift count K = min(e_hi, m-1), once, and 1 for the count of each
+    threshold; for reads that no stripes hold the linear form, per word of 32
+    bases 3, 15 per step and 6 per threshold."""
     K = min(e_hi, max(m - 1, 0))
-    return S * (4 + 10 * K + (e_hi - e_lo + 1))
+    S = stripes_of(m)
+    if S:
+        return S * (4 + 10 * K + (e_hi - e_lo + 1))
+    return -(-m // 32) * (3 + 15 * K + 6 * (e_hi - e_lo + 1))
+
+
+def form_ops_per_pair(m, K, striped, overlap, shared):
+    """ALU operations per pair at one shift count K in the form that the
+    library runs, from which a launch's share of the integer peak follows: per
+    word 3 for the first mask's difference and dilation and 6 for the final
+    erosion and count, and per step 8 striped (S words), 7 and the read's 4
+    funnel shifts in overlapping words, 11 and those 4 in words side by side
+    (``shared``: two pairs of one read, 2 of the 4 each); exact erosion above
+    30, and without one of the forms, 22."""
+    W = -(-m // 32)
+    if K > 30:
+        return W * (13 + 22 * K)
+    if striped:
+        return stripes_of(m) * (9 + 8 * K)
+    return W * (9 + K * ((7 if overlap else 11) + (2 if shared else 4)))
+
+
+def single_ops_per_pair(m: int, e: int) -> float:
+    """form_ops_per_pair of the form that gk_filter runs one threshold in."""
+    W, K = -(-m // 32), min(e, max(m - 1, 0))
+    if K < 2 and W > 4:
+        return W * (13 + 22 * K)
+    overlap = 2 <= W <= 8 and m <= 30 * W and K <= 7 and (W != 5 or K >= 3)
+    start = {6: 16, 7: 9, 9: 14, 10: 12}.get(W, 8)
+    striped = not overlap and 3 <= W <= 10 and K >= start and stripes_of(m) == (W if W <= 5 else 8 if W <= 8 else 11)
+    return form_ops_per_pair(m, K, striped, overlap, W <= 4)
+
+
+def batched_ops_per_pair(m: int, e: int) -> float:
+    """form_ops_per_pair of a batched launch's one pair per lane."""
+    W, K = -(-m // 32), min(e, m - 1)
+    start = {4: 8, 5: 11, 7: 14, 8: 10}.get(W, 31)
+    return form_ops_per_pair(m, K, K >= start and stripes_of(m) == (W if W <= 5 else 8), False, False)
 
 
 def pp_sweep_bytes_per_pair(m: int, c: float, n_thresholds: int, result_byte: bool = False) -> float:
@@ -536,17 +581,17 @@ def run_mine(args):
     peak_basis = f"{SM_COUNT} SMs x {ALU_LANES_PER_SM_CLK:.0f} int lanes/clk x {SM_MAX_MHZ:.0f} MHz"
 
     def per_pair_roofline(per_e_ms):
-        """Word formulation: algorithmic ops per launch summed over the sweep,
-        over the summed CUDA-event durations of those launches."""
-        ops = sum(w.n_pairs * ops_per_pair(m, e) for e in E_SWEEP)
+        """The launches' operations in the form each runs (single_ops_per_pair)
+        summed over the sweep, over their summed CUDA-event durations."""
+        ops = sum(w.n_pairs * single_ops_per_pair(m, e) for e in E_SWEEP)
         tops = ops / (sum(per_e_ms) * 1e-3) / 1e12
         bpp = bytes_per_pair(m, c, False)
         gbs = w.n_pairs * bpp * len(E_SWEEP) / (sum(per_e_ms) * 1e-3) / 1e9
         # Per threshold: the launch against the slower of its bytes at the
-        # HBM peak and its word-formulation ops at the integer peak.
+        # HBM peak and its form's ops at the integer peak.
         per_e = {}
         for e, ms in zip(E_SWEEP, per_e_ms):
-            ceil = min(hbm_peak * 1e9 / bpp, ALU_PEAK_TOPS * 1e12 / ops_per_pair(m, e))
+            ceil = min(hbm_peak * 1e9 / bpp, ALU_PEAK_TOPS * 1e12 / single_ops_per_pair(m, e))
             rate = w.n_pairs / (ms * 1e-3)
             per_e[str(e)] = {"gpairs_s": rate / 1e9, "roofline_gpairs_s": ceil / 1e9, "frac": rate / ceil}
         return {"bound": "alu", "achieved": tops, "peak": ALU_PEAK_TOPS, "unit": "Tops/s",
@@ -554,7 +599,8 @@ def run_mine(args):
                 "kernel": ("filter_pair2_kernel<W, 4, K, -1> (e 0-2, two pairs per thread, shift count fixed at "
                            "compile time) | filter_pair2_kernel<W, 2, -1, S> (e 3-10: overlapping words, striped "
                            "from 8)"),
-                "ops_basis": "W*(9 + 22e + 4) per pair (word formulation)", "peak_basis": peak_basis,
+                "ops_basis": "single_ops_per_pair: the operations of the form that each threshold runs in",
+                "peak_basis": peak_basis,
                 "bytes_side": {"achieved_gbs": gbs, "peak_gbs": hbm_peak, "frac": gbs / hbm_peak,
                                "bytes_per_pair": bpp},
                 "per_e_of_roofline": per_e}
@@ -967,11 +1013,11 @@ def measure_c3(args, hbm_peak: float) -> dict:
         undefined = int((dd.edits_u16(ed) == gk.GK_EDITS_UNDEFINED).sum())
         filtered = n - undefined
         pp_ms = sum(per_e.values())
-        pp_ops = sum(filtered * ops_per_pair(m, e) for e in es)
+        pp_ops = sum(filtered * single_ops_per_pair(m, e) for e in es)
         per_pair = {"gpairs_s": n * len(es) / (pp_ms * 1e-3) / 1e9, "ms": pp_ms,
                     "per_e_gpairs_s": {str(e): n / (t * 1e-3) / 1e9 for e, t in per_e.items()},
                     "alu_frac": pp_ops / (pp_ms * 1e-3) / 1e12 / ALU_PEAK_TOPS,
-                    "alu_basis": "W(13 + 22e) per filtered (non-N) pair, word formulation",
+                    "alu_basis": "single_ops_per_pair per filtered (non-N) pair",
                     "survey_bytes_frac": n * bytes_per_pair(m, c, False) * len(es) / (pp_ms * 1e-3) / 1e9 / hbm_peak}
         # per-pair sweep: one launch for every threshold
         psa = torch.empty(len(es) * n, dtype=torch.uint8, device="cuda")
@@ -983,7 +1029,7 @@ def measure_c3(args, hbm_peak: float) -> dict:
         pp_sweep = {"gpairs_s": n * len(es) / (ps_ms * 1e-3) / 1e9, "ms": ps_ms,
                     "form": f"one gk_filter_sweep over e {es[0]}..{es[-1]}",
                     "alu_frac": ps_ops / (ps_ms * 1e-3) / 1e12 / ALU_PEAK_TOPS,
-                    "alu_basis": "W(9 + 22K + 4 n_thresholds) per filtered (non-N) pair, K = min(e_hi, m-1)",
+                    "alu_basis": "pp_sweep_ops_per_pair per filtered (non-N) pair: S(4 + 10K + n_thresholds)",
                     "bytes_frac": n * pp_sweep_bytes_per_pair(m, c, len(es)) / (ps_ms * 1e-3) / 1e9 / hbm_peak,
                     "survey_bytes_frac": n * bytes_per_pair(m, c, False) * len(es) / (ps_ms * 1e-3) / 1e9 / hbm_peak}
         del psa, pse
@@ -1033,8 +1079,8 @@ def measure_c3(args, hbm_peak: float) -> dict:
 
 def measure_c4(args) -> dict:
     """Config 4: 50M pairs, lengths U{50..300}, per-pair e = ceil(rate m),
-    shuffled: one graph-captured gk_filter_batched (classify, scan, scatter,
-    persistent filter) with the autotuner's tiling, against the plain filter
+    shuffled: one graph-captured gk_filter_batched (pairs sorted into records,
+    a filter launch per range of lengths) with the autotuner's tiling, against the plain filter
     launched once per read length over the same pairs."""
     import torch
 
@@ -1053,7 +1099,8 @@ def measure_c4(args) -> dict:
     results = {}
     if args.tune_seconds > 0:  # autotune on a seeded sample of the pairs
         rng = np.random.default_rng(3)
-        samp = np.sort(rng.choice(w.n_pairs, min(w.n_pairs, 4_000_000), replace=False))
+        # Above 8M pairs, as the whole is: one filter launch per range of lengths.
+        samp = np.sort(rng.choice(w.n_pairs, min(w.n_pairs, 9_000_000), replace=False))
         sp = dd.upload_pairs(w.pair_read[samp], w.pair_off[samp], w.pair_e[samp])
         best, results = batch.autotune(ref, reads.packed, reads.stride_words, reads.n_reads, read_len,
                                        reads.nflag, sp.pair_read, sp.pair_off, sp.pair_e, reps=2,
@@ -1090,21 +1137,20 @@ def measure_c4(args) -> dict:
     torch.cuda.synchronize()
     inv = torch.from_numpy(np.argsort(order))
     same = bool(torch.equal(acc.cpu()[inv], bf.accept.cpu()) and torch.equal(ed.cpu()[inv], bf.edits.cpu()))
-    Wp = (m_pair.astype(np.int64) + 31) // 32
-    ek = np.minimum(w.pair_e.astype(np.int64), m_pair.astype(np.int64) - 1)
-    ops = float(np.sum(Wp * (13 + 22 * ek)))
+    key, count = np.unique(m_pair.astype(np.int64) * 256 + w.pair_e, return_counts=True)
+    ops = float(sum(n * batched_ops_per_pair(int(k) // 256, int(k) % 256) for k, n in zip(key, count)))
     ref.close()
     return {
         "value": w.n_pairs / (batched_ms * 1e-3) / 1e9, "unit": "Gpairs/s", "ms": batched_ms, "steps": steps,
-        "pairs": w.n_pairs, "form": "one CUDA-graph replay of gk_filter_batched (classify, scan, scatter, "
-                                    "persistent filter)",
+        "pairs": w.n_pairs, "form": "one CUDA-graph replay of gk_filter_batched (words_per_thread 1: "
+                                    "records sorted by clusters, one filter launch per range of lengths)",
         "tiling": {"words_per_thread": best[0], "tile_pairs": best[1], "blocks_per_sm": best[2],
-                   "warps_per_block": best[3], "source": "autotuned on a 4M-pair sample" if results else "table"},
+                   "warps_per_block": best[3], "source": "autotuned on a 9M-pair sample" if results else "table"},
         "autotune_candidates_ms": {",".join(map(str, k)): v for k, v in results.items()},
         "plain_per_length": {"value": w.n_pairs / (plain_ms * 1e-3) / 1e9, "ms": plain_ms,
                              "launches": int(len(starts)), "identical_results": same},
         "alu_frac": ops / (batched_ms * 1e-3) / 1e12 / ALU_PEAK_TOPS,
-        "alu_basis": "W(13 + 22 min(e, m-1)) per pair, word formulation, over the whole graph",
+        "alu_basis": "batched_ops_per_pair per pair, over the whole graph",
         "generation_s": t_gen}
 
 
