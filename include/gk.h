@@ -316,7 +316,7 @@ uint64_t gk_filter_batched_workspace(uint64_t n_pairs);
 
 /*
  * gk_filter_batched -- filter pairs of mixed read lengths and per-pair
- * thresholds in one persistent launch (the paper batches many reads and their
+ * thresholds in one call (the paper batches many reads and their
  * candidates per kernel call, Sec. 3.3 and Sec. 3.5; same per-pair result as
  * gk_filter, Sec. 2.1/3.3/3.4).
  *

@@ -752,14 +752,15 @@ __device__ __forceinline__ uint32_t filter_loaded_deferred(const FilterArgs &a, 
   return count[0];
 }
 
-// Resident blocks per SM the compiler must allow.  One thread per pair:
-// small reads keep enough registers free for 40 warps per SM, which hides
-// the dependent loads of a pair (ids, then read and window words); W = 5 and
-// 6 fit 4 and 3 blocks without spilling (at 150 bp, e = 0..2, 4 blocks run
-// 9-18% faster than 2).  The compacting loop stages its words with cp.async
-// and carries a chunk pipeline, so it keeps fewer resident warps.
-// The striped sweep needs 56 (S <= 4), 72 (S = 5), 93 (S = 8) and 128 (S =
-// 11) registers.
+// Resident blocks per SM the compiler must allow: of 256 threads in the
+// compacting loop, of 128 elsewhere.  One thread per pair: small reads keep
+// enough registers free for 40 warps per SM, which hides the dependent loads
+// of a pair (ids, then read and window words); W = 5 and 6 fit 32 and 24 warps
+// without spilling (at 150 bp, e = 0..2, 32 warps run 9-18% faster than 16).
+// The compacting loop stages its words with cp.async and carries a chunk
+// pipeline, so it keeps fewer resident warps.
+// The striped loops use 64 registers (S <= 4), 80 (S = 5), 91 (S = 8; 128 in
+// the compacting loop) and 128 (S = 11).
 template <int W, bool COMPACT, int S = 0>
 struct MinBlocks {
   static constexpr int value =
@@ -1133,8 +1134,8 @@ __global__ void __launch_bounds__(COMPACT ? kQueueThreads : kFilterThreads, MinB
 // slower at every other shift count at 100 bp.
 constexpr bool kPair2Wide = false;
 
-// Resident blocks per SM of the two-pairs-per-thread kernel: 4 (64 registers,
-// a few spilled) measured faster than 3 (80 registers, no spill) at every
+// Resident blocks of 128 threads per SM of the two-pairs-per-thread kernel: 8
+// (64 registers, a few spilled) measured faster than 6 (80 registers, no spill) at every
 // threshold 1..10 and in the 0..10 sweep at 100 bp on GB300 (e = 2: 53.3 ->
 // 57.5 Gpairs/s; the sweep 1.307 -> 1.280 ms), the same at e = 0.
 template <int W>

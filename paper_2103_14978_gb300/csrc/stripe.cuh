@@ -24,7 +24,7 @@
 //                   and lies outside the read (m <= 32 S - 4).
 //
 // S is the smallest of these that holds the read: 32 S positions, 2 (even) or
-// 4 (odd) of them to spare.  Every step is bound by the integer ALU pipe (88-93% busy):
+// 4 (odd) of them to spare.  Every step is bound by the integer ALU pipe (81-88% busy):
 // logic ops and right shifts run there at 64 lanes per clock and SM, left
 // shifts and additions partly on the multiply-add pipe, which is why the
 // vectors below move up (to higher positions) wherever there is a choice.
@@ -295,7 +295,7 @@ __host__ __device__ __forceinline__ uint32_t stripe_count(const uint32_t (&f)[S]
 // Measured on GB300 against the linear sweep, launches alone: 20M pairs of 100
 // bp at e = 0..10 1.206 -> 0.744 ms; 5M pairs of 150 bp at 0..15 0.548 -> 0.350
 // ms, of 250 bp at 0..25 1.334 -> 0.844 ms; ALU operations per pair at 100 bp
-// 1088 -> 680.  With the logic ops left to the compiler's own 3-input merging
+// 1088 -> 651.  With the logic ops left to the compiler's own 3-input merging
 // the step took 7 more of them (0.799 ms): it shares x[w] & x[w-1] between
 // neighbours first, hence lop3.
 template <int W, int S, int NP, bool WHOLE, typename Emit>

@@ -430,7 +430,7 @@ def gk_filter_batched(ref: Reference, reads: torch.Tensor, stride_words: int, n_
                       pair_off: torch.Tensor, e, tiling: Tiling, workspace: torch.Tensor,
                       count_mode: int = GK_COUNT_RUNS4, flags: int = 0, accept: torch.Tensor | None = None,
                       edits: torch.Tensor | None = None, err_count: torch.Tensor | None = None, stream=None):
-    """Filter pairs of mixed read lengths in one persistent launch
+    """Filter pairs of mixed read lengths in one call
     (gk_filter_batched).  ``read_len`` is an int16 CUDA tensor (uint16
     values); ``workspace`` a uint8 CUDA tensor of at least
     gk_filter_batched_workspace(n) bytes.  Returns (accept, edits); with
