@@ -23,10 +23,10 @@
 // 1.15 of 5.3 ms for 50M pairs.
 //
 // Measured on GB300 against that sort, 50M pairs of 50-300 bp, per-pair
-// thresholds of 2, 5 and 10%, random order: 5.29 -> 4.61 ms per graph launch
+// thresholds of 2, 5 and 10%, random order: 5.30 -> 4.53 ms per graph launch
 // (planning 0.81, bound by the gathers of read length and N flag; the filters by
 // the ALU pipe, those of up to 128 bp by the gathers of shuffled read rows); a
-// server round of 3M pairs of 100, 150 and 250 bp (three calls) 0.392 -> 0.248
+// server round of 3M pairs of 100, 150 and 250 bp (three calls) 0.400 -> 0.241
 // ms.  9M pairs of 36-512 bp 1.97 -> 2.11, of 200-512 bp 2.70 -> 2.78: a launch
 // above 8M pairs whose rows have more than 10 words is the slower one.
 #pragma once
